@@ -1,8 +1,12 @@
 // tcgen05 BF16 / FP8-e4m3 candidate search for the cosine KNN of Section 3.1.
 //
-// Persistent CTAs (one per SM) share the (128-row query block, 256-row key
-// tile) pairs in equal contiguous runs (stream-K), so no wave tail is left
-// idle.  In each CTA:
+// Two kernels share one scheme.  k_knn_pair sweeps all keys with CTA pairs
+// (every full sweep); k_knn_tc, one CTA at a time, takes the sweeps of listed
+// key tiles, of a sample of the tiles and of keys above a threshold.
+//
+// Persistent CTAs (one per SM) share the (query block, 256-row key tile)
+// pairs in equal contiguous runs (stream-K), so no wave tail is left idle.
+// In each CTA of k_knn_tc:
 //   warp 0     TMA producer: the current query block A (128 x dp, 128-byte
 //              swizzle) when the run enters it, then key tiles B (256 rows x
 //              128 bytes of features per stage: 64 BF16 or 128 FP8) through
@@ -24,6 +28,12 @@
 // leave the SM.  Every mbarrier wait is bounded: on expiry the kernel records
 // an error code, stops all roles, drains its own copies and MMAs (bounded),
 // frees TMEM and returns.
+//
+// The producer and the MMA issuer run their loops as whole warps and elect a
+// lane for the copies, MMAs and commits alone.  With the loops inside one
+// lane's branch the MMAs, whose operands want uniform registers, took 167
+// cycles each and a stage's hand-off another 160; warp-uniform they take 130,
+// the tensor pipe's own rate (M = 256 over a pair, N = 256, K = 16).
 #include <algorithm>
 #include <atomic>
 
@@ -111,32 +121,74 @@ __device__ __forceinline__ float pick32(const uint32_t (&r)[32], int e) {
     for (int q = 0; q < w; ++q) v[q] = (e & w) ? v[q + w] : v[q];
   return v[0];
 }
-
-// Fold one 32-key chunk (scores in r, keys j0..j0+31, mx = their maximum
-// from the TMEM load) into the row's list.
-template <int C>
-__device__ __forceinline__ void fold_chunk(const uint32_t (&r)[32], float mx, int64_t j0, int64_t n, int64_t i,
-                                           float (&lv)[C], int32_t (&li)[C]) {
-  // skip the chunk when no lane of the warp has a key above its threshold
-  const float thr0 = lv[C - 1];
-  if (!__any_sync(0xffffffffu, mx > thr0)) return;
-  // pass mask against the threshold at chunk start (it only rises, so the
-  // mask is a superset); padding keys and the row itself removed
-  uint32_t pm = 0;
+// the same over 16
+__device__ __forceinline__ float pick16(const uint32_t (&r)[16], int e) {
+  float v[8];
 #pragma unroll
-  for (int e = 0; e < 32; ++e) pm |= (__uint_as_float(r[e]) > thr0 ? 1u : 0u) << e;
-  if (j0 + 32 > n) pm &= (j0 >= n) ? 0u : ((1u << (uint32_t)(n - j0)) - 1u);
-  if (i >= j0 && i < j0 + 32) pm &= ~(1u << (uint32_t)(i - j0));
-  // one insert per passing key; lanes without keys idle
-  while (__any_sync(0xffffffffu, pm != 0)) {
-    if (pm) {
+  for (int q = 0; q < 8; ++q) v[q] = __uint_as_float((e & 8) ? r[q + 8] : r[q]);
+#pragma unroll
+  for (int w = 4; w >= 1; w >>= 1)
+#pragma unroll
+    for (int q = 0; q < w; ++q) v[q] = (e & w) ? v[q + w] : v[q];
+  return v[0];
+}
+
+// A row's list, and a 16-key chunk with a key above the threshold that has
+// not been looked into yet (pj == kNoChunk: none).  Finding and inserting a
+// key costs the whole warp ~150 dependent instructions however few lanes need
+// it, so a lane that meets such a chunk sets it aside, 16 moves, and the warp
+// goes through its lanes' chunks together once some lane has a second one
+// (after about seven).  The threshold lags by the chunk, which only lets more
+// keys through to the insert's own test: the list is the same.
+constexpr uint32_t kNoChunk = 0xffffffffu;
+template <int C>
+struct RowList {
+  float lv[C];
+  int32_t li[C];
+  uint32_t pr[16];  // the chunk's scores
+  uint32_t pj;      // its first key
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      lv[c] = -INFINITY;
+      li[c] = -1;
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) pr[e] = 0;
+    pj = kNoChunk;
+  }
+  // the warp's chunks into its lists; n keys, i: the key this row excludes
+  // (itself), or -1
+  __device__ __forceinline__ void flush(uint32_t n, uint32_t i) {
+    // pass mask against the threshold now (it only rises, so the mask is a
+    // superset), in four chains; padding keys and the row itself removed
+    const float thr = lv[C - 1];
+    uint32_t q[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int e = 0; e < 16; ++e) q[e & 3] |= (__uint_as_float(pr[e]) > thr ? 1u : 0u) << e;
+    uint32_t pm = pj == kNoChunk ? 0u : (q[0] | q[1]) | (q[2] | q[3]);
+    if (pj < n && n - pj < 16) pm &= (1u << (n - pj)) - 1u;
+    if (pj >= n) pm = 0;
+    if (i - pj < 16) pm &= ~(1u << (i - pj));
+    // one key per lane and round; lanes without keys idle
+    while (__any_sync(0xffffffffu, pm != 0)) {
       const int e = __ffs(pm) - 1;
+      const float v = pick16(pr, e);
+      if (pm != 0 && v > lv[C - 1]) sorted_insert<C>(lv, li, v, (int32_t)(pj + e));
       pm &= pm - 1;
-      const float val = pick32(r, e);
-      if (val > lv[C - 1]) sorted_insert<C>(lv, li, val, (int32_t)(j0 + e));
+    }
+    pj = kNoChunk;
+  }
+  // set aside the chunk r (keys j0 ..) in the lanes whose maximum of it passes
+  __device__ __forceinline__ void push(const uint32_t (&r)[16], float mx, uint32_t j0, uint32_t n, uint32_t i) {
+    if (__any_sync(0xffffffffu, mx > lv[C - 1] && pj != kNoChunk)) flush(n, i);
+    if (mx > lv[C - 1]) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) pr[e] = r[e];
+      pj = j0;
     }
   }
-}
+};
 
 // Collect mode: append every key whose score reaches the row's fixed
 // threshold t to the row's buffer (cap entries; the counter keeps counting
@@ -155,6 +207,40 @@ __device__ __forceinline__ void collect_chunk(const uint32_t (&r)[32], float mx,
     pm &= pm - 1;
     const int pos = atomicAdd(&cnt[ra], 1);
     if (pos < cap) buf[ra * (int64_t)cap + pos] = (int32_t)(j0 + e);
+  }
+}
+
+// Fold one tile's column slice (kSliceN accumulator columns from TMEM address
+// tb, keys jb ...) into the row's list, 64 columns at a time (all 128 would
+// not fit the registers of 10 warps): four 16-column loads with the
+// hardware's maximum of each behind one wait, then four independent votes
+// that say which chunks hold a key above some lane's threshold (two of the
+// tile's eight at n = 600,000).  release() hands the accumulator back once
+// the last column has landed, before the list work on it.
+template <int C, int kPart, class Release>
+__device__ __forceinline__ void fold_slice(uint32_t tb, uint32_t jb, uint32_t n, uint32_t i, RowList<C>& L,
+                                           Release&& release) {
+#pragma unroll 1
+  for (int p = 0; p < kSliceN; p += 16 * kPart) {
+    uint32_t r[kPart][16];
+    float mx[kPart];
+#pragma unroll
+    for (int c = 0; c < kPart; ++c) tmem_ld16_max_issue(tb + (uint32_t)(p + c * 16), r[c], mx[c]);
+    tmem_wait();
+#pragma unroll
+    for (int c = 0; c < kPart; ++c) {
+      pin(r[c]);
+      pin1(mx[c]);
+    }
+    if (p + 16 * kPart == kSliceN) release();
+    const float thr = L.lv[C - 1];
+    uint32_t hit = 0;
+#pragma unroll
+    for (int c = 0; c < kPart; ++c) hit |= (__any_sync(0xffffffffu, mx[c] > thr) ? 1u : 0u) << c;
+    if (hit == 0) continue;
+#pragma unroll
+    for (int c = 0; c < kPart; ++c)
+      if (hit & (1u << c)) L.push(r[c], mx[c], jb + (uint32_t)(p + c * 16), n, i);
   }
 }
 
@@ -244,7 +330,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
   uint8_t* sA = smem;
   uint8_t* sB = sA + kb_count * kABytes;
   Bars* bars = reinterpret_cast<Bars*>(sB + nstages * kBBytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
   const int n_tiles = (int)ceil_div(ceil_div(n_pad, kTN), key_stride);
   const int64_t work = ca.blk_ptr ? ca.blk_work : qblocks * n_tiles;
   const int64_t w_begin = range_begin(blockIdx.x, work, gridDim.x);
@@ -279,123 +365,133 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
   const uint32_t tmem = bars->tmem_base;
 
   if (warp == 0) {
-    if (lane == 0) {
-      bool pending[kMaxStages];
-      uint32_t pend_par[kMaxStages];
-      for (int s = 0; s < kMaxStages; ++s) pending[s] = false;
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      int seg = 0;
-      uint32_t tiles_issued = 0;
-      for (int64_t w = w_begin; w < w_end && ok; ++seg) {
-        const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
-        const int64_t qb = sg.qb;
-        const int t0 = sg.t0, t1 = sg.t1;
-        int rot = ca.blk_ptr ? 0 : key_rotation(qb, n_tiles, work, gridDim.x);
-        w += t1 - t0;
-        // the previous block of A stays in use until its last MMA completes
-        if (seg > 0 && !mbar_wait(&bars->a_empty, (uint32_t)((seg - 1) & 1), abort, err, 6)) {
-          ok = false;
-          break;
-        }
-        // A block this CTA sweeps whole starts at the key tile the CTAs are
-        // reading now (tiles issued by all CTAs / CTAs), so that CTAs whose
-        // rates drift apart re-align at every block and keep sharing the key
-        // tiles in L2; a split block keeps the static rotation both of its
-        // CTAs can compute.
-        if (tick && !ca.blk_ptr && t0 == 0 && t1 == n_tiles)
-          rot = (int)((*reinterpret_cast<volatile unsigned long long*>(tick) / gridDim.x) % (uint64_t)n_tiles);
+    bool pending[kMaxStages];
+    uint32_t pend_par[kMaxStages];
+    for (int s = 0; s < kMaxStages; ++s) pending[s] = false;
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int seg = 0;
+    uint32_t tiles_issued = 0;
+    const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+    for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+      const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
+      const int64_t qb = sg.qb;
+      const int t0 = sg.t0, t1 = sg.t1;
+      int rot = ca.blk_ptr ? 0 : key_rotation(qb, n_tiles, work, gridDim.x);
+      w += t1 - t0;
+      // the previous block of A stays in use until its last MMA completes
+      if (seg > 0 && !mbar_wait_warp(&bars->a_empty, (uint32_t)((seg - 1) & 1), abort, err, 6)) {
+        ok = false;
+        break;
+      }
+      // A block this CTA sweeps whole starts at the key tile the CTAs are
+      // reading now (tiles issued by all CTAs / CTAs), so that CTAs whose
+      // rates drift apart re-align at every block and keep sharing the key
+      // tiles in L2; a split block keeps the static rotation both of its
+      // CTAs can compute.
+      if (tick && !ca.blk_ptr && t0 == 0 && t1 == n_tiles)
+        rot = (int)((*reinterpret_cast<volatile unsigned long long*>(tick) / gridDim.x) % (uint64_t)n_tiles);
+      rot = __shfl_sync(0xffffffffu, rot, 0);
+      if (elect_one()) {
         bars->rot[seg & 1] = rot;
         __threadfence_block();
         mbar_expect_tx(&bars->a_full, (uint32_t)(kb_count * kABytes));
         for (int kb = 0; kb < kb_count; ++kb)
-          tma_load_2d(smem_u32(sA + kb * kABytes), &tmA, kb * kTK, (int)(qb * kTM), &bars->a_full);
-        for (int t = t0; t < t1 && ok; ++t) {
-          for (int kb = 0; kb < kb_count; ++kb) {
-            if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort, err, 1)) {
-              ok = false;
-              break;
-            }
-            pending[stage] = false;
-            mbar_expect_tx(&bars->full[stage], (uint32_t)kBBytes);
-            const int kt = ca.blk_ptr ? ca.blk_tiles[sg.base + t]
-                                      : (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * key_stride;
-            tma_load_2d(smem_u32(sB + stage * kBBytes), &tmB, kb * kTK, kt * kTN, &bars->full[stage]);
-            pending[stage] = true;
-            pend_par[stage] = phase;
-            if (++stage == nstages) {
-              stage = 0;
-              phase ^= 1;
-            }
-          }
-          if (tick && ((++tiles_issued) & 15) == 0) atomicAdd(tick, 16ull);
-        }
+          tma_load_2d(sA0 + kb * kABytes, &tmA, kb * kTK, (int)(qb * kTM), &bars->a_full);
       }
-      if (!ok) {  // drain this warp's copies still in flight (bounded)
-        if (seg > 0) mbar_wait(&bars->a_full, (uint32_t)((seg - 1) & 1), nullptr, nullptr, 0);
-        for (int s = 0; s < nstages; ++s)
-          if (pending[s]) mbar_wait(&bars->full[s], pend_par[s], nullptr, nullptr, 0);
+      __syncwarp();
+      for (int t = t0; t < t1 && ok; ++t) {
+        const int kt = ca.blk_ptr ? ca.blk_tiles[sg.base + t]
+                                  : (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * key_stride;
+        for (int kb = 0; kb < kb_count; ++kb) {
+          if (!mbar_wait_warp(&bars->empty[stage], phase ^ 1, abort, err, 1)) {
+            ok = false;
+            break;
+          }
+          if (elect_one()) {
+            mbar_expect_tx(&bars->full[stage], (uint32_t)kBBytes);
+            tma_load_2d(sB0 + stage * kBBytes, &tmB, kb * kTK, kt * kTN, &bars->full[stage]);
+          }
+          __syncwarp();
+          pending[stage] = true;
+          pend_par[stage] = phase;
+          if (++stage == nstages) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
+        if (tick && ((++tiles_issued) & 15) == 0 && lane == 0) atomicAdd(tick, 16ull);
       }
     }
+    if (!ok) {  // drain this warp's copies still in flight (bounded)
+      if (seg > 0) mbar_wait(&bars->a_full, (uint32_t)((seg - 1) & 1), nullptr, nullptr, 0);
+      for (int s = 0; s < nstages; ++s)
+        if (pending[s]) mbar_wait(&bars->full[s], pend_par[s], nullptr, nullptr, 0);
+    }
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = true;
-      int stage = 0;
-      uint32_t phase = 0;
-      bool issued = false;
-      int64_t g = 0;  // accumulator tiles so far (ping-pong over two)
-      int seg = 0;
-      for (int64_t w = w_begin; w < w_end && ok; ++seg) {
-        const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
-        const int t0 = sg.t0, t1 = sg.t1;
-        w += t1 - t0;
-        if (!mbar_wait(&bars->a_full, (uint32_t)(seg & 1), abort, err, 2)) {
+    bool ok = true;
+    int stage = 0;
+    uint32_t phase = 0;
+    bool issued = false;
+    int64_t g = 0;  // accumulator tiles so far (ping-pong over two)
+    int seg = 0;
+    const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+    for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+      const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
+      const int t0 = sg.t0, t1 = sg.t1;
+      w += t1 - t0;
+      if (!mbar_wait_warp(&bars->a_full, (uint32_t)(seg & 1), abort, err, 2)) {
+        ok = false;
+        break;
+      }
+      for (int t = t0; t < t1; ++t, ++g) {
+        const int b = (int)(g & 1);
+        const uint32_t use = (uint32_t)(g >> 1);
+        if (!mbar_wait_warp(&bars->tempty[b], (use & 1) ^ 1, abort, err, 3)) {
           ok = false;
           break;
         }
-        for (int t = t0; t < t1; ++t, ++g) {
-          const int b = (int)(g & 1);
-          const uint32_t use = (uint32_t)(g >> 1);
-          if (!mbar_wait(&bars->tempty[b], (use & 1) ^ 1, abort, err, 3)) {
+        tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)(b * kTN);
+        for (int kb = 0; kb < kb_count; ++kb) {
+          if (!mbar_wait_warp(&bars->full[stage], phase, abort, err, 4)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t d = tmem + (uint32_t)(b * kTN);
-          for (int kb = 0; kb < kb_count; ++kb) {
-            if (!mbar_wait(&bars->full[stage], phase, abort, err, 4)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t a0 = smem_u32(sA + kb * kABytes);
-            const uint32_t b0 = smem_u32(sB + stage * kBBytes);
-            const int kmax = kb == kb_count - 1 ? k_last : kMmaPerStage;
+          const uint64_t a0 = sw128_desc(sA0 + kb * kABytes);
+          const uint64_t b0 = sw128_desc(sB0 + stage * kBBytes);
+          const int kmax = kb == kb_count - 1 ? k_last : kMmaPerStage;
+          if (elect_one()) {
+            // the next 32 bytes of K: 2 more in the descriptors' 16-byte units
 #pragma unroll
-            for (int kk = 0; kk < kMmaPerStage; ++kk) {
-              if (kk >= kmax) break;
-              if constexpr (kE4M3)
-                umma_e4m3(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), (kb | kk) != 0 ? 1u : 0u);
-              else
-                umma_bf16(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), (kb | kk) != 0 ? 1u : 0u);
-            }
-            issued = true;
+            for (int kk = 0; kk < kMmaPerStage; ++kk)
+              if (kk < kmax) {
+                if constexpr (kE4M3)
+                  umma_e4m3(d, a0 + kk * 2, b0 + kk * 2, (kb | kk) != 0 ? 1u : 0u);
+                else
+                  umma_bf16(d, a0 + kk * 2, b0 + kk * 2, (kb | kk) != 0 ? 1u : 0u);
+              }
             umma_commit(&bars->empty[stage]);
-            if (++stage == nstages) {
-              stage = 0;
-              phase ^= 1;
-            }
+            if (kb == kb_count - 1) umma_commit(&bars->tfull[b]);
           }
-          if (!ok) break;
-          umma_commit(&bars->tfull[b]);
+          __syncwarp();
+          issued = true;
+          if (++stage == nstages) {
+            stage = 0;
+            phase ^= 1;
+          }
         }
-        if (ok) umma_commit(&bars->a_empty);  // A may be replaced once these MMAs complete
+        if (!ok) break;
       }
-      if (!ok && issued) {  // wait for this thread's MMAs before TMEM is freed (bounded)
-        umma_commit(&bars->drain);
-        mbar_wait(&bars->drain, 0, nullptr, nullptr, 0);
-      }
+      if (ok && elect_one()) umma_commit(&bars->a_empty);  // A may be replaced once these MMAs complete
+      __syncwarp();
+    }
+    if (!ok && issued) {  // wait for the MMAs issued before TMEM is freed (bounded)
+      if (elect_one()) umma_commit(&bars->drain);
+      __syncwarp();
+      mbar_wait(&bars->drain, 0, nullptr, nullptr, 0);
     }
   } else {
     const int ew = warp - 2;   // epilogue warp 0..7
@@ -420,13 +516,8 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
       const int64_t i = ca.a_rows ? (row_ok ? (int64_t)ca.a_rows[ra] : -1) : ra;
       const int64_t i_self = ca.no_self ? -1 : i;  // the key index this row excludes
       const float t_row = kCollect && row_ok ? ca.thr[ra] : INFINITY;
-      float lv[C];
-      int32_t li[C];
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        lv[c] = -INFINITY;
-        li[c] = -1;
-      }
+      RowList<C> L;
+      L.clear();
       for (int t = t0; t < t1; ++t, ++g) {
         const int b = (int)(g & 1);
         const uint32_t use = (uint32_t)(g >> 1);
@@ -443,29 +534,33 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                                   : (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * key_stride;
         const int64_t jb = (int64_t)kt * kTN + h * kSliceN;
         const uint32_t tb = lane_base + (uint32_t)(b * kTN + h * kSliceN);
-        // the hardware's maximum over each 32-column load settles most
-        // chunks with one compare and one vote
+        // the hardware's maximum over each load settles most chunks with one
+        // compare and one vote
+        auto release = [&] {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->tempty[b]);
+        };
+        if constexpr (kCollect) {
 #pragma unroll 1
-        for (int c = 0; c < kSliceN / 32; ++c) {
-          uint32_t rv[32];
-          float mx;
-          tmem_ld32_max_issue(tb + (uint32_t)(c * 32), rv, mx);
-          tmem_wait();
-          pin(rv);
-          pin1(mx);
-          if constexpr (kCollect) {
+          for (int c = 0; c < kSliceN / 32; ++c) {
+            uint32_t rv[32];
+            float mx;
+            tmem_ld32_max_issue(tb + (uint32_t)(c * 32), rv, mx);
+            tmem_wait();
+            pin(rv);
+            pin1(mx);
             collect_chunk(rv, mx, jb + c * 32, n, i_self, t_row, ra, ca.cnt, ca.buf, ca.cap);
-          } else {
-            fold_chunk<C>(rv, mx, jb + c * 32, n, i_self, lv, li);
           }
+          release();
+        } else {
+          fold_slice<C, 4>(tb, (uint32_t)jb, (uint32_t)n, (uint32_t)i_self, L, release);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->tempty[b]);
       }
       if (!kCollect && ok) {
         float* ov;
         int32_t* oi;
+        L.flush((uint32_t)n, (uint32_t)i_self);
         if (t0 == 0 && t1 == sg.len) {  // whole block: final lists
           if (!row_ok) continue;
           ov = cand_val + i * kCandC;
@@ -477,8 +572,8 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         }
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          ov[h * C + c] = lv[c] * sc;
-          oi[h * C + c] = li[c];
+          ov[h * C + c] = L.lv[c] * sc;
+          oi[h * C + c] = L.li[c];
         }
       }
     }
@@ -491,59 +586,440 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
   }
 }
 
+// ---------------------------------------------------------------------------
+// Full sweep on CTA pairs.
+//
+// A CTA that sweeps alone reads 12 KB of shared memory per 128 x 256 x 16 MMA
+// and writes 8 KB (9 KB at d = 100) of key tiles for it, more than the 128
+// bytes a cycle its shared memory gives in the 128 cycles that MMA takes.  Two
+// CTAs of a cluster (the two SMs of a TPC) therefore share one M = 256,
+// N = 256 accumulator pair (tcgen05 cta_group::2): each holds its own 128
+// query rows and half (128) of a tile's keys, so that per MMA an SM reads
+// 8 KB and writes 4 KB, and the key bytes that come from L2 halve.
+//
+// Measured (the contraction with its row preparation, one CTA a sweep before,
+// the pair now): 72 -> 46.0 ms at n = 600,000, d = 100 (bound by the MMAs'
+// power draw and the list work; 41 ms without the list work); 6.9 -> 5.2 ms
+// at n = 100,000, d = 500 (MMA bound: 4150 cycles a tile for 32 MMAs, SM clock
+// 1.8 GHz under power); E4M3 3.4 -> 2.55 ms at n = 100,003, d = 256 (list
+// work: 1.7 ms without it).
+//
+// Roles as in k_knn_tc, in both CTAs, except that the even CTA (the leader)
+// alone issues the MMAs.  Each CTA's producer loads its own half and signals
+// the leader's barrier (cta_group::2 copies), which expects the bytes of
+// both; the commits of the leader's MMAs arrive in both CTAs (multicast), and
+// the epilogue warps of both release an accumulator at the leader's barrier.
+// The unit of work is 256 query rows x 256 keys, split stream-K over the
+// pairs.  The leader picks a block's key rotation and hands it to its peer.
+// ---------------------------------------------------------------------------
+constexpr int kPairRows = 2 * kTM;             // query rows of a pair's block
+constexpr int kPairBBytes = kTN / 2 * kTKB;    // 16 KB of keys per stage and CTA
+constexpr int kPairMaxStages = 12;
+// Three warpgroups: the producer, the MMA issuer and two idle warps, then the
+// eight epilogue warps.  What decides whether the MMAs wait is how soon an
+// accumulator comes back, so the epilogue takes all 128 columns of its slice
+// into registers before it looks at them; the first warpgroup gives up its
+// registers for that (setmaxnreg: 128 x 64 + 256 x 216 = 63,488 of the
+// 384 x 168 = 64,512 the block is launched with).
+constexpr int kPairThreads = 128 + 32 * kEpiWarps;
+constexpr int kPairRegsLow = 64, kPairRegsHigh = 216;
+
+struct __align__(8) PairBars {
+  uint64_t full[kPairMaxStages];   // leader: both CTAs' halves of the stage have landed
+  uint64_t empty[kPairMaxStages];  // each CTA: the MMAs that read the stage have completed
+  uint64_t a_full;                 // leader: both CTAs' query rows have landed
+  uint64_t a_empty;                // each CTA
+  uint64_t tfull[2];               // each CTA
+  uint64_t tempty[2];              // leader: released by the epilogue warps of both
+  uint64_t rot_full;               // peer: the leader has written rot
+  uint64_t drain;
+  uint32_t tmem_base;
+  int abort;
+  int rot[2];  // key rotation of the current and the previous segment
+};
+
+// M = 256 over the pair
+constexpr uint32_t kIdescPairBF16 = (kIdescBF16 & ~(0x1fu << 24)) | ((uint32_t)(kPairRows >> 4) << 24);
+constexpr uint32_t kIdescPairE4M3 = (kIdescE4M3 & ~(0x1fu << 24)) | ((uint32_t)(kPairRows >> 4) << 24);
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+  __syncwarp();
+}
+// this CTA's shared address as CTA `rank`'s address at the same offset
+__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void pair_tma_load(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+      "[%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
+      : "memory");
+}
+template <bool kE4M3>
+__device__ __forceinline__ void pair_umma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t accum) {
+  if constexpr (kE4M3)
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, "
+        "p;\n}" ::"r"(tmem_d),
+        "l"(da), "l"(db), "r"(kIdescPairE4M3), "r"(accum)
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
+            tmem_d),
+        "l"(da), "l"(db), "r"(kIdescPairBF16), "r"(accum)
+        : "memory");
+}
+// arrives at the barrier's offset in both CTAs once this thread's MMAs complete
+__device__ __forceinline__ void pair_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void pair_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// One CTA of the pair; grid = 2 x pairs.  Arguments as for k_knn_tc; part_*
+// hold two slots of kPairRows rows per pair.
+template <bool kE4M3>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
+           int64_t n_pad, int64_t qblocks, int kb_count, int k_last, int nstages, float* __restrict__ cand_val,
+           int32_t* __restrict__ cand_idx, const float* __restrict__ out_scale, float* __restrict__ part_val,
+           int32_t* __restrict__ part_idx, const int32_t* __restrict__ a_rows, int64_t n_rows,
+           unsigned long long* __restrict__ tick, int* __restrict__ err) {
+  constexpr int kTK = kE4M3 ? 128 : 64;  // features per stage
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sA = smem;
+  uint8_t* sB = sA + kb_count * kABytes;
+  PairBars* bars = reinterpret_cast<PairBars*>(sB + nstages * kPairBBytes);
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
+  const uint32_t rank = cluster_rank();
+  const bool leader = rank == 0;
+  const int64_t pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  const int n_tiles = (int)ceil_div(n_pad, kTN);
+  const int64_t work = qblocks * n_tiles;
+  const int64_t w_begin = range_begin(pair, work, pairs);
+  const int64_t w_end = range_begin(pair + 1, work, pairs);
+  const CollectArgs none{};
+  volatile int* abort = &bars->abort;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < nstages; ++s) {
+      mbar_init(&bars->full[s], 1);
+      mbar_init(&bars->empty[s], 1);
+    }
+    mbar_init(&bars->a_full, 1);
+    mbar_init(&bars->a_empty, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&bars->tfull[b], 1);
+      mbar_init(&bars->tempty[b], 2 * kEpiWarps);
+    }
+    mbar_init(&bars->rot_full, 1);
+    mbar_init(&bars->drain, 1);
+    bars->abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&bars->tmem_base)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // both CTAs' barriers and TMEM are ready
+  tc_fence_after();
+  const uint32_t tmem = bars->tmem_base;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPairRegsLow));
+    if (warp == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      int seg = 0;
+      uint32_t tiles_issued = 0;
+      const uint32_t a_full = peer_addr(smem_u32(&bars->a_full), 0);
+      const uint32_t full0 = peer_addr(smem_u32(&bars->full[0]), 0);
+      const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+      for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+        const Seg sg = segment_at(w, w_end, n_tiles, qblocks, none);
+        w += sg.t1 - sg.t0;
+        // the previous query rows stay in use until their last MMA completes
+        if (seg > 0 && !mbar_wait_warp(&bars->a_empty, (uint32_t)((seg - 1) & 1), abort, err, 6)) {
+          ok = false;
+          break;
+        }
+        // Key order: as in k_knn_tc, a block the pair sweeps whole starts at
+        // the tile the pairs are reading now, a split block at the static
+        // rotation both of its pairs compute.
+        int rot;
+        if (leader) {
+          rot = key_rotation(sg.qb, n_tiles, work, pairs);
+          if (sg.t0 == 0 && sg.t1 == n_tiles)
+            rot = (int)((*reinterpret_cast<volatile unsigned long long*>(tick) / pairs) % (uint64_t)n_tiles);
+          rot = __shfl_sync(0xffffffffu, rot, 0);
+          if (elect_one()) {
+            bars->rot[seg & 1] = rot;
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(smem_u32(&bars->rot[seg & 1]), 1)), "r"(rot)
+                         : "memory");
+            asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                             peer_addr(smem_u32(&bars->rot_full), 1))
+                         : "memory");
+          }
+        } else {
+          if (!mbar_wait_warp(&bars->rot_full, (uint32_t)(seg & 1), abort, err, 7)) {
+            ok = false;
+            break;
+          }
+          asm volatile("fence.acq_rel.cluster;" ::: "memory");
+          rot = *reinterpret_cast<volatile int*>(&bars->rot[seg & 1]);
+          rot = __shfl_sync(0xffffffffu, rot, 0);
+        }
+        if (elect_one()) {
+          if (leader) mbar_expect_tx(&bars->a_full, (uint32_t)(2 * kb_count * kABytes));
+          for (int kb = 0; kb < kb_count; ++kb)
+            pair_tma_load(sA0 + kb * kABytes, &tmA, kb * kTK, (int)(sg.qb * kPairRows + rank * kTM), a_full);
+        }
+        __syncwarp();
+        for (int t = sg.t0; t < sg.t1 && ok; ++t) {
+          const int kt = t + rot < n_tiles ? t + rot : t + rot - n_tiles;
+          for (int kb = 0; kb < kb_count; ++kb) {
+            if (!mbar_wait_warp(&bars->empty[stage], phase ^ 1, abort, err, 1)) {
+              ok = false;
+              break;
+            }
+            if (elect_one()) {
+              if (leader) mbar_expect_tx(&bars->full[stage], (uint32_t)(2 * kPairBBytes));
+              pair_tma_load(sB0 + stage * kPairBBytes, &tmB, kb * kTK, (int)(kt * kTN + rank * (kTN / 2)),
+                            full0 + (uint32_t)(stage * sizeof(uint64_t)));
+            }
+            __syncwarp();
+            if (++stage == nstages) {
+              stage = 0;
+              phase ^= 1;
+            }
+          }
+          if (leader && ((++tiles_issued) & 15) == 0 && lane == 0) atomicAdd(tick, 16ull);
+        }
+      }
+      // on an abort, let this CTA's copies in flight land before the CTA may
+      // exit: they report to the leader's barriers, so a fixed time (~1 ms,
+      // several hundred times a copy's latency) stands in for a wait on them
+      if (!ok)
+        for (const long long t0 = clock64(); clock64() - t0 < 2000000;) {
+        }
+    } else if (warp == 1) {
+      if (leader) {
+        bool ok = true;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool issued = false;
+        int64_t g = 0;  // accumulator tiles so far (ping-pong over two)
+        int seg = 0;
+        const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+        for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+          const Seg sg = segment_at(w, w_end, n_tiles, qblocks, none);
+          w += sg.t1 - sg.t0;
+          if (!mbar_wait_warp(&bars->a_full, (uint32_t)(seg & 1), abort, err, 2)) {
+            ok = false;
+            break;
+          }
+          for (int t = sg.t0; t < sg.t1; ++t, ++g) {
+            const int b = (int)(g & 1);
+            const uint32_t use = (uint32_t)(g >> 1);
+            if (!mbar_wait_warp(&bars->tempty[b], (use & 1) ^ 1, abort, err, 3)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)(b * kTN);
+            for (int kb = 0; kb < kb_count; ++kb) {
+              if (!mbar_wait_warp(&bars->full[stage], phase, abort, err, 4)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint64_t a0 = sw128_desc(sA0 + kb * kABytes);
+              const uint64_t b0 = sw128_desc(sB0 + stage * kPairBBytes);
+              const int kmax = kb == kb_count - 1 ? k_last : kMmaPerStage;
+              if (elect_one()) {
+                // the next 32 bytes of K: 2 more in the descriptors' 16-byte units
+  #pragma unroll
+                for (int kk = 0; kk < kMmaPerStage; ++kk)
+                  if (kk < kmax) pair_umma<kE4M3>(d, a0 + kk * 2, b0 + kk * 2, (kb | kk) != 0 ? 1u : 0u);
+                pair_commit(&bars->empty[stage]);
+                if (kb == kb_count - 1) pair_commit(&bars->tfull[b]);
+              }
+              __syncwarp();
+              issued = true;
+              if (++stage == nstages) {
+                stage = 0;
+                phase ^= 1;
+              }
+            }
+            if (!ok) break;
+          }
+          if (ok && elect_one()) pair_commit(&bars->a_empty);  // the query rows may be replaced once these MMAs complete
+          __syncwarp();
+        }
+        if (!ok && issued) {  // wait for this thread's MMAs before TMEM is freed (bounded)
+          if (elect_one()) pair_commit(&bars->drain);
+          __syncwarp();
+          mbar_wait(&bars->drain, 0, nullptr, nullptr, 0);
+        }
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPairRegsHigh));
+    const int q = warp & 3;          // TMEM lane quarter this warp may access
+    const int h = (warp - 4) >> 2;   // column half of every tile
+    const int r = q * 32 + lane;
+    constexpr int C = kListC;
+    const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * kSliceN);
+    const float sc = out_scale ? *out_scale : 1.f;
+    const uint32_t tempty0 = peer_addr(smem_u32(&bars->tempty[0]), 0);
+    int64_t g = 0;
+    int seg = 0;
+    bool ok = true;
+    for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+      const Seg sg = segment_at(w, w_end, n_tiles, qblocks, none);
+      int rot = 0;
+      w += sg.t1 - sg.t0;
+      const int64_t ra = sg.qb * kPairRows + rank * kTM + r;
+      const bool row_ok = ra < n_rows;
+      const int64_t i = a_rows ? (row_ok ? (int64_t)a_rows[ra] : -1) : ra;
+      RowList<C> L;
+      L.clear();
+      for (int t = sg.t0; t < sg.t1; ++t, ++g) {
+        const int b = (int)(g & 1);
+        const bool got = mbar_wait(&bars->tfull[b], (uint32_t)(g >> 1) & 1u, abort, err, 5);
+        if (!__all_sync(0xffffffffu, got)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        // written before the segment's query rows were loaded, which its
+        // first accumulator waited for
+        if (t == sg.t0) rot = *reinterpret_cast<volatile int*>(&bars->rot[seg & 1]);
+        const int kt = t + rot < n_tiles ? t + rot : t + rot - n_tiles;
+        const uint32_t jb = (uint32_t)kt * kTN + (uint32_t)(h * kSliceN);
+        const uint32_t tb = lane_base + (uint32_t)(b * kTN);
+        auto release = [&] {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) pair_arrive(tempty0 + (uint32_t)(b * sizeof(uint64_t)));
+        };
+        fold_slice<C, 8>(tb, jb, (uint32_t)n, (uint32_t)i, L, release);
+      }
+      if (!ok) break;
+      L.flush((uint32_t)n, (uint32_t)i);
+      float* ov;
+      int32_t* oi;
+      if (sg.t0 == 0 && sg.t1 == n_tiles) {  // whole block: final lists
+        if (!row_ok) continue;
+        ov = cand_val + i * kCandC;
+        oi = cand_idx + i * kCandC;
+      } else {
+        const int64_t slot = (pair * 2 + (seg == 0 ? 0 : 1)) * kPairRows + rank * kTM + r;
+        ov = part_val + slot * kCandC;
+        oi = part_idx + slot * kCandC;
+      }
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        ov[h * C + c] = L.lv[c] * sc;
+        oi[h * C + c] = L.li[c];
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // no CTA leaves while its peer may still signal it or read its keys
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+}
+
 // Lists of the query blocks split between runs: per row and column half, the
 // 16 best of the pieces' lists (each piece holds the best of its own key
-// tiles, so the result is the best of the whole half).  One CTA of kTM
-// threads per query block; blocks that one run covered return at once.
+// tiles, so the result is the best of the whole half).  One CTA per query
+// block, one thread per row (kRows: 128, or 256 for pairs) and half; blocks
+// that one run covered return at once.  A piece's 16 entries are loaded
+// together: with one entry at a time and both halves in one thread, the eight
+// pieces a block has at n = 2000 took 80 us of a call of 185 us.
 // Block qb's work items are [x0, x1) = [qb n_tiles, (qb + 1) n_tiles), or
 // [blk_ptr[qb], blk_ptr[qb + 1]) in tile-list mode (a block with no tiles
 // gets empty lists).
-__global__ void __launch_bounds__(kTM) k_merge_lists(int n_tiles, int64_t work, int64_t ctas,
-                                                     const int64_t* __restrict__ blk_ptr,
-                                                     const float* __restrict__ part_val,
-                                                     const int32_t* __restrict__ part_idx,
-                                                     const int32_t* __restrict__ a_rows, int64_t n_rows,
-                                                     float* __restrict__ cand_val, int32_t* __restrict__ cand_idx) {
+template <int kRows>
+__global__ void __launch_bounds__(2 * kRows)
+k_merge_lists(int n_tiles, int64_t work, int64_t ctas, const int64_t* __restrict__ blk_ptr,
+              const float* __restrict__ part_val, const int32_t* __restrict__ part_idx,
+              const int32_t* __restrict__ a_rows, int64_t n_rows, float* __restrict__ cand_val,
+              int32_t* __restrict__ cand_idx) {
+  static_assert(kLists == 2 && kListC == 16, "a thread per half, four 16-byte loads per list");
   const int64_t qb = blockIdx.x;
   const int64_t x0 = blk_ptr ? blk_ptr[qb] : qb * n_tiles;
   const int64_t x1 = blk_ptr ? blk_ptr[qb + 1] : x0 + n_tiles;
-  const int r = threadIdx.x;
-  const int64_t ra = qb * kTM + r;
+  const int r = threadIdx.x % kRows, h = threadIdx.x / kRows;
+  const int64_t ra = qb * kRows + r;
   if (ra >= n_rows) return;
   const int64_t i = a_rows ? (int64_t)a_rows[ra] : ra;
   constexpr int C = kListC;
-  if (x0 == x1) {
-    for (int e = 0; e < kCandC; ++e) {
-      cand_val[i * kCandC + e] = -INFINITY;
-      cand_idx[i * kCandC + e] = -1;
-    }
-    return;
-  }
-  const int64_t c0 = ((x0 + 1) * ctas + work - 1) / work - 1;  // the CTA whose range holds x0
-  if (range_begin(c0 + 1, work, ctas) >= x1) return;
-  for (int h = 0; h < kLists; ++h) {
-    float lv[C];
-    int32_t li[C];
+  float* ov = cand_val + i * kCandC + h * C;
+  int32_t* oi = cand_idx + i * kCandC + h * C;
+  float lv[C];
+  int32_t li[C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      lv[c] = -INFINITY;
-      li[c] = -1;
-    }
+  for (int c = 0; c < C; ++c) {
+    lv[c] = -INFINITY;
+    li[c] = -1;
+  }
+  if (x0 < x1) {
+    const int64_t c0 = ((x0 + 1) * ctas + work - 1) / work - 1;  // the CTA whose range holds x0
+    if (range_begin(c0 + 1, work, ctas) >= x1) return;           // covered whole: its lists are final
     for (int64_t cc = c0; cc < ctas; ++cc) {
       const int64_t b = range_begin(cc, work, ctas);
       if (b >= x1) break;
-      const int64_t slot = (cc * 2 + (b >= x0 ? 0 : 1)) * kTM + r;  // run cc starts inside the block: its first segment
+      const int64_t slot = (cc * 2 + (b >= x0 ? 0 : 1)) * kRows + r;  // run cc starts inside the block: its first segment
+      const float4* pv = reinterpret_cast<const float4*>(part_val + slot * kCandC + h * C);
+      const int4* pi = reinterpret_cast<const int4*>(part_idx + slot * kCandC + h * C);
+      float v[C];
+      int32_t j[C];
+#pragma unroll
+      for (int q = 0; q < C / 4; ++q) {
+        const float4 f = pv[q];
+        const int4 g = pi[q];
+        v[4 * q] = f.x, v[4 * q + 1] = f.y, v[4 * q + 2] = f.z, v[4 * q + 3] = f.w;
+        j[4 * q] = g.x, j[4 * q + 1] = g.y, j[4 * q + 2] = g.z, j[4 * q + 3] = g.w;
+      }
+      // the piece is sorted: nothing after its first entry that does not pass can pass
+#pragma unroll
       for (int e = 0; e < C; ++e) {
-        const int32_t j = part_idx[slot * kCandC + h * C + e];
-        const float v = part_val[slot * kCandC + h * C + e];
-        if (j >= 0 && v > lv[C - 1]) sorted_insert<C>(lv, li, v, j);
+        if (!(j[e] >= 0 && v[e] > lv[C - 1])) break;
+        sorted_insert<C>(lv, li, v[e], j[e]);
       }
     }
+  }
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      cand_val[i * kCandC + h * C + c] = lv[c];
-      cand_idx[i * kCandC + h * C + c] = li[c];
-    }
+  for (int q = 0; q < C / 4; ++q) {
+    reinterpret_cast<float4*>(ov)[q] = make_float4(lv[4 * q], lv[4 * q + 1], lv[4 * q + 2], lv[4 * q + 3]);
+    reinterpret_cast<int4*>(oi)[q] = make_int4(li[4 * q], li[4 * q + 1], li[4 * q + 2], li[4 * q + 3]);
   }
 }
 
@@ -1025,10 +1501,50 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
                                                                    out_scale, part_val, part_idx, ca, tick, err);
   ANCKA_LAUNCHED();
   if (!kCollect) {
-    k_merge_lists<<<(unsigned)qblocks, kTM, 0, s>>>(n_tiles, work, ctas, ca.blk_ptr, part_val, part_idx, ca.a_rows,
+    k_merge_lists<kTM><<<(unsigned)qblocks, 2 * kTM, 0, s>>>(n_tiles, work, ctas, ca.blk_ptr, part_val, part_idx, ca.a_rows,
                                                     n_rows, cand_val, cand_idx);
     ANCKA_LAUNCHED();
   }
+  return ANCKA_OK;
+}
+
+// The full sweep by CTA pairs: every row's two lists over all keys (rows of
+// a_rows, written at their own row index, or rows 0..n-1).
+template <bool kE4M3>
+ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& tb, int64_t n, int64_t n_pad,
+                         const int32_t* a_rows, int64_t n_rows, int kb_count, int d, float* cand_val,
+                         int32_t* cand_idx, const float* out_scale, int32_t* err, cudaStream_t s) {
+  const int per_kb = kE4M3 ? 128 : 64, per_mma = kE4M3 ? 32 : 16;  // k_last as in launch_tc
+  const int rem = d - per_kb * (kb_count - 1);
+  const int k_last = (rem >= 1 && rem <= per_kb) ? (int)ceil_div(rem, per_mma) : kMmaPerStage;
+  const size_t fixed = 1024 + (size_t)kb_count * kABytes + sizeof(PairBars);
+  const int nstages = (int)std::min<size_t>(kPairMaxStages, (kMaxSmem - fixed) / kPairBBytes);
+  const size_t smem = fixed + (size_t)nstages * kPairBBytes;  // > 120 KB for every kb_count: one CTA per SM
+  if (nstages < 4) {
+    set_error("tensor-core contraction: not enough shared memory for four stages");
+    return ANCKA_ERR_UNSUPPORTED;
+  }
+  int sms = 152, dev = 0;
+  ANCKA_CUDA(cudaGetDevice(&dev));
+  ANCKA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int64_t qblocks = ceil_div(n_rows, kPairRows);
+  const int n_tiles = (int)ceil_div(n_pad, kTN);
+  const int64_t work = qblocks * n_tiles;
+  const int64_t pairs = std::max<int64_t>(1, std::min<int64_t>(sms / 2, work));
+  float* part_val;
+  int32_t* part_idx;
+  unsigned long long* tick;
+  ANCKA_TRY(ws.alloc(&part_val, (size_t)pairs * 2 * kPairRows * kCandC));
+  ANCKA_TRY(ws.alloc(&part_idx, (size_t)pairs * 2 * kPairRows * kCandC));
+  ANCKA_TRY(ws.zeros(&tick, 1));
+  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_pair<kE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_knn_pair<kE4M3><<<(unsigned)(2 * pairs), kPairThreads, smem, s>>>(
+      ta, tb, n, n_pad, qblocks, kb_count, k_last, nstages, cand_val, cand_idx, out_scale, part_val, part_idx,
+      a_rows, n_rows, tick, err);
+  ANCKA_LAUNCHED();
+  k_merge_lists<kPairRows><<<(unsigned)qblocks, 2 * kPairRows, 0, s>>>(n_tiles, work, pairs, nullptr, part_val, part_idx,
+                                                                   a_rows, n_rows, cand_val, cand_idx);
+  ANCKA_LAUNCHED();
   return ANCKA_OK;
 }
 
@@ -1115,12 +1631,12 @@ ancka_status knn_candidates_bf16(Workspace& ws, const PrepOut& pr, int64_t n, fl
   }
   CUtensorMap ta, tb;
   ANCKA_TRY(make_map(&ta, pr.xb, pr.dp, pr.n_pad, kTM, 2));
-  ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN, 2));
-  if (n >= g_sym_min_rows.load(std::memory_order_relaxed))
+  if (n >= g_sym_min_rows.load(std::memory_order_relaxed)) {
+    ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN, 2));
     return knn_candidates_bf16_sym(ws, pr, n, ta, tb, kb_count, cand_val, cand_idx, err, s);
-  CollectArgs none{};
-  return launch_tc<false, false>(ws, ta, tb, n, pr.n_pad, n, kb_count, pr.d, cand_val, cand_idx, nullptr, none, err,
-                                 s);
+  }
+  ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN / 2, 2));
+  return launch_pair<false>(ws, ta, tb, n, pr.n_pad, nullptr, n, kb_count, pr.d, cand_val, cand_idx, nullptr, err, s);
 }
 
 void knn_set_symmetric_min_rows(int64_t n_min) { g_sym_min_rows.store(n_min, std::memory_order_relaxed); }
@@ -1134,10 +1650,8 @@ ancka_status knn_candidates_fp8(Workspace& ws, const PrepOut& pr, int64_t n, flo
   }
   CUtensorMap ta, tb;
   ANCKA_TRY(make_map(&ta, pr.x8, pr.dp8, pr.n_pad, kTM, 1));
-  ANCKA_TRY(make_map(&tb, pr.x8, pr.dp8, pr.n_pad, kTN, 1));
-  CollectArgs none{};
-  return launch_tc<false, true>(ws, ta, tb, n, pr.n_pad, n, kb_count, pr.d, cand_val, cand_idx, pr.inv_s2, none, err,
-                                s);
+  ANCKA_TRY(make_map(&tb, pr.x8, pr.dp8, pr.n_pad, kTN / 2, 1));
+  return launch_pair<true>(ws, ta, tb, n, pr.n_pad, nullptr, n, kb_count, pr.d, cand_val, cand_idx, pr.inv_s2, err, s);
 }
 
 int knn_tc_max_dp_fp8() { return 1024; }
@@ -1154,10 +1668,8 @@ ancka_status knn_list_gathered_bf16(Workspace& ws, const PrepOut& pr, int64_t n,
   ANCKA_LAUNCHED();
   CUtensorMap ta, tb;
   ANCKA_TRY(make_map(&ta, af, pr.dp, n_a_pad, kTM, 2));
-  ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN, 2));
-  CollectArgs ca{rows, n_a, nullptr, nullptr, nullptr, 0};
-  return launch_tc<false, false>(ws, ta, tb, n, pr.n_pad, n_a, kb_count, pr.d, cand_val, cand_idx, nullptr, ca, err,
-                                 s);
+  ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN / 2, 2));
+  return launch_pair<false>(ws, ta, tb, n, pr.n_pad, rows, n_a, kb_count, pr.d, cand_val, cand_idx, nullptr, err, s);
 }
 
 ancka_status knn_lists_bf16(Workspace& ws, const __nv_bfloat16* a, int64_t a_rows_total, const int32_t* rows,

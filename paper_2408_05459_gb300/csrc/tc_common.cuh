@@ -36,7 +36,7 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
 }
 // bounded wait; false on expiry (which raises the CTA-wide abort) or when
 // another role has already aborted
-__device__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort, int* err, int code) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort, int* err, int code) {
   if (mbar_try(b, parity)) return true;
   const long long t0 = clock64();
   while (true) {
@@ -48,6 +48,29 @@ __device__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort, int
       return false;
     }
   }
+}
+
+// The same by a whole converged warp, so that the roles' loops stay
+// warp-uniform: their addresses and descriptors are then kept in uniform
+// registers, where the copy and MMA instructions want them.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort, int* err, int code) {
+  if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;
+  const long long t0 = clock64();
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;
+    if (__any_sync(0xffffffffu, abort && *abort)) return false;
+    if (__any_sync(0xffffffffu, clock64() - t0 > kWaitCycles)) {
+      if (abort) *abort = 1;
+      if (err) atomicExch(err, code);
+      return false;
+    }
+  }
+}
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e != 0;
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
@@ -102,12 +125,23 @@ __device__ __forceinline__ void tmem_ld32_max_issue(uint32_t taddr, uint32_t (&r
         "=f"(mx)
       : "r"(taddr));
 }
+// the 16-column form
+__device__ __forceinline__ void tmem_ld16_max_issue(uint32_t taddr, uint32_t (&r)[16], float& mx) {
+  asm volatile(
+      "tcgen05.ld.red.sync.aligned.32x32b.x16.max.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+      "%14, %15}, %16, [%17];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=f"(mx)
+      : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void pin1(float& x) { asm volatile("" : "+f"(x)); }
 // make every later use of r depend on this point (after the wait)
-__device__ __forceinline__ void pin(uint32_t (&r)[32]) {
+template <int N>
+__device__ __forceinline__ void pin(uint32_t (&r)[N]) {
 #pragma unroll
-  for (int q = 0; q < 32; ++q) asm volatile("" : "+r"(r[q]));
+  for (int q = 0; q < N; ++q) asm volatile("" : "+r"(r[q]));
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
