@@ -29,7 +29,10 @@ namespace ancka {
 
 namespace {
 
-constexpr int kIvfChunk = 4096;  // rows per chunk of the counting sort
+// Rows per chunk of the counting sort: a warp places a chunk 32 rows at a
+// time, so short chunks put more warps to work; the chunks' table of nlist
+// positions each stays below about 4 bytes a row and 32 MB per 2^20 rows.
+inline int ivf_chunk(int nlist) { return nlist <= 1024 ? 1024 : 4096; }
 constexpr int kTileRows = 256;   // key rows per tile of the contraction
 constexpr int kBlockRows = 128;  // query rows per block of the contraction
 
@@ -78,101 +81,146 @@ __global__ void k_ivf_top(const float* __restrict__ cand_val, const int32_t* __r
 // counting sort of a sequence of rows (seq, or the rows in order) by a key
 // per row (cell), stable: per-chunk histograms ...
 __global__ void k_ivf_hist(const int32_t* __restrict__ cell, const int32_t* __restrict__ seq, int64_t n, int nlist,
-                           int32_t* __restrict__ hist) {
+                           int chunk, int32_t* __restrict__ hist) {
   const int64_t ch = blockIdx.x;
-  const int64_t r0 = ch * kIvfChunk, r1 = min(n, r0 + kIvfChunk);
+  const int64_t r0 = ch * chunk, r1 = min(n, r0 + chunk);
   for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x)
     atomicAdd(&hist[ch * nlist + max(0, cell[seq ? seq[r] : r])], 1);
 }
 
-// ... per cell, the chunks' offsets inside the cell and the cell's size ...
+// ... per cell, the chunks' offsets inside the cell and the cell's size (a
+// warp per cell, 32 chunks at a time) ...
 __global__ void k_ivf_cell_scan(int32_t* __restrict__ hist, int64_t nchunks, int nlist,
                                 int64_t* __restrict__ cell_size) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
   if (l >= nlist) return;
   int64_t run = 0;
-  for (int64_t ch = 0; ch < nchunks; ++ch) {
-    const int32_t c = hist[ch * nlist + l];
-    hist[ch * nlist + l] = (int32_t)run;
-    run += c;
+  for (int64_t c0 = 0; c0 < nchunks; c0 += 32) {
+    const int64_t ch = c0 + lane;
+    const int32_t c = ch < nchunks ? hist[ch * nlist + l] : 0;
+    int32_t x = c;
+    for (int off = 1; off < 32; off <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, x, off);
+      if (lane >= off) x += y;
+    }
+    if (ch < nchunks) hist[ch * nlist + l] = (int32_t)(run + x - c);
+    run += __shfl_sync(0xffffffffu, x, 31);
   }
-  cell_size[l] = run;
+  if (lane == 0) cell_size[l] = run;
 }
 
-// ... exclusive scan of the cell sizes (one CTA, fixed order) ...
-__global__ void k_ivf_exscan(const int64_t* __restrict__ in, int count, int64_t* __restrict__ out) {
-  __shared__ int64_t part[1024];
-  const int t = threadIdx.x, per = (count + blockDim.x - 1) / blockDim.x;
-  const int a = t * per, b = min(count, a + per);
+// ... exclusive scan of the cell sizes (one CTA of 1024 threads) ...
+__global__ void __launch_bounds__(1024) k_ivf_exscan(const int64_t* __restrict__ in, int count,
+                                                     int64_t* __restrict__ out) {
+  __shared__ int64_t wtot[32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, per = (count + blockDim.x - 1) / blockDim.x;
+  const int a = min(count, t * per), b = min(count, a + per);
   int64_t s = 0;
   for (int e = a; e < b; ++e) s += in[e];
-  part[t] = s;
+  int64_t x = s;
+  for (int off = 1; off < 32; off <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
+  }
+  if (lane == 31) wtot[w] = x;
   __syncthreads();
-  if (t == 0) {
-    int64_t run = 0;
-    for (int u = 0; u < (int)blockDim.x; ++u) {
-      const int64_t v = part[u];
-      part[u] = run;
-      run += v;
+  if (w == 0) {
+    int64_t y = wtot[lane];
+    for (int off = 1; off < 32; off <<= 1) {
+      const int64_t z = __shfl_up_sync(0xffffffffu, y, off);
+      if (lane >= off) y += z;
     }
-    out[count] = run;
+    wtot[lane] = y;
   }
   __syncthreads();
-  int64_t run = part[t];
+  int64_t run = x - s + (w > 0 ? wtot[w - 1] : 0);
   for (int e = a; e < b; ++e) {
     out[e] = run;
     run += in[e];
   }
+  if (t == 0) out[count] = wtot[31];
 }
 
-// ... and the placement: a chunk's rows in sequence order (one thread per chunk)
-__global__ void k_ivf_place(const int32_t* __restrict__ cell, const int32_t* __restrict__ seq, int64_t n, int nlist,
-                            int32_t* __restrict__ hist, const int64_t* __restrict__ cell_off,
-                            int32_t* __restrict__ order) {
-  const int64_t ch = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t r0 = ch * kIvfChunk;
-  if (r0 >= n) return;
-  const int64_t r1 = min(n, r0 + kIvfChunk);
-  // the chunk's running position per cell lives in global scratch: the
-  // offsets table row of this chunk is advanced in place (each chunk owns it)
-  int32_t* pos = hist + ch * nlist;
-  for (int64_t r = r0; r < r1; ++r) {
-    const int32_t row = seq ? seq[r] : (int32_t)r;
-    const int l = max(0, cell[row]);  // a row with no finite score (NaN input) joins cell 0
-    order[cell_off[l] + pos[l]++] = row;
-  }
-}
-
-// centroid = normalised sum of its members' unit rows (one warp per cell,
-// members in row order, FP32); an empty cell keeps its centroid
-__global__ void k_ivf_update(const __nv_bfloat16* __restrict__ xb, int dp, const int32_t* __restrict__ order,
-                             const int64_t* __restrict__ cell_off, int nlist, __nv_bfloat16* __restrict__ C) {
-  const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (l >= nlist) return;
-  const int64_t a = cell_off[l], b = cell_off[l + 1];
-  if (a == b) return;
-  float acc[16];
+// ... and the placement, a warp per chunk, 32 rows of the sequence at a time:
+// rows of the same cell are ranked by lane, which keeps their order, and the
+// first of them advances the cell's position, held in shared memory.  (One
+// thread per chunk, reading and advancing its positions in global memory row
+// by row, was a chain of 4096 round trips: 0.68 ms a sort on average over the ten
+// of a call at n = 600,000 and 500 cells, 16 us now.)
+constexpr int kPlaceBatch = 4;  // rounds whose rows and cells are loaded together
+__global__ void __launch_bounds__(32)
+k_ivf_place(const int32_t* __restrict__ cell, const int32_t* __restrict__ seq, int64_t n, int nlist, int chunk,
+            const int32_t* __restrict__ hist, const int64_t* __restrict__ cell_off, int32_t* __restrict__ order) {
+  extern __shared__ int32_t pos[];
+  const int lane = threadIdx.x;
+  const int64_t ch = blockIdx.x;
+  const int64_t r0 = ch * chunk, r1 = min(n, r0 + chunk);
+  for (int l = lane; l < nlist; l += 32) pos[l] = hist[ch * nlist + l] + (int32_t)cell_off[l];  // < n < 2^31
+  __syncwarp();
+  for (int64_t rb = r0; rb < r1; rb += 32 * kPlaceBatch) {
+    int32_t row[kPlaceBatch], cl[kPlaceBatch];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) acc[q] = 0.f;
-  for (int64_t p = a; p < b; ++p) {
-    const __nv_bfloat16* row = xb + (int64_t)order[p] * dp;
+    for (int q = 0; q < kPlaceBatch; ++q) {
+      const int64_t r = rb + 32 * q + lane;
+      row[q] = r < r1 ? (seq ? seq[r] : (int32_t)r) : -1;
+    }
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int f = lane + 32 * q;
-      if (f < dp) acc[q] += __bfloat162float(row[f]);
+    for (int q = 0; q < kPlaceBatch; ++q)
+      cl[q] = row[q] >= 0 ? max(0, cell[row[q]]) : -1;  // a row with no finite score (NaN input) joins cell 0
+#pragma unroll
+    for (int q = 0; q < kPlaceBatch; ++q) {
+      const unsigned peers = __match_any_sync(0xffffffffu, cl[q]);
+      const int first = __ffs(peers) - 1;
+      int32_t base = 0;
+      if (lane == first && cl[q] >= 0) {
+        base = pos[cl[q]];
+        pos[cl[q]] = base + __popc(peers);
+      }
+      base = __shfl_sync(0xffffffffu, base, first);
+      if (cl[q] >= 0) order[base + __popc(peers & ((1u << lane) - 1u))] = row[q];
+      __syncwarp();
     }
   }
-  float ss = 0.f;
+}
+
+// centroid = normalised sum of its members' unit rows (members in row order,
+// FP32); an empty cell keeps its centroid.  A CTA per cell, a warp per 32
+// features, 16 members' loads in flight (a warp per cell with one member's
+// loads in flight was latency bound: 177 us a launch at 500 cells, dp = 128,
+// 47 us now).
+constexpr int kUpdateBatch = 16;
+__global__ void k_ivf_update(const __nv_bfloat16* __restrict__ xb, int dp, const int32_t* __restrict__ order,
+                             const int64_t* __restrict__ cell_off, int nlist, __nv_bfloat16* __restrict__ C) {
+  __shared__ float sums[512];
+  __shared__ float sinv;
+  const int l = blockIdx.x;
+  const int f = threadIdx.x;  // blockDim.x = dp
+  const int64_t a = cell_off[l], b = cell_off[l + 1];
+  if (a == b) return;
+  float acc = 0.f;
+  for (int64_t p = a; p < b; p += kUpdateBatch) {
+    int32_t row[kUpdateBatch];
+    __nv_bfloat16 v[kUpdateBatch];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) ss = fmaf(acc[q], acc[q], ss);
-  for (int off = 16; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-  const float inv = ss > 0.f ? rsqrtf(ss) : 0.f;
+    for (int q = 0; q < kUpdateBatch; ++q) row[q] = p + q < b ? order[p + q] : -1;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const int f = lane + 32 * q;
-    if (f < dp) C[(int64_t)l * dp + f] = __float2bfloat16(acc[q] * inv);
+    for (int q = 0; q < kUpdateBatch; ++q)
+      if (row[q] >= 0) v[q] = xb[(int64_t)row[q] * dp + f];
+#pragma unroll
+    for (int q = 0; q < kUpdateBatch; ++q)
+      if (row[q] >= 0) acc += __bfloat162float(v[q]);
   }
+  sums[f] = acc;
+  __syncthreads();
+  if (f < 32) {
+    float ss = 0.f;
+    for (int c = f; c < dp; c += 32) ss = fmaf(sums[c], sums[c], ss);
+    for (int off = 16; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+    if (f == 0) sinv = ss > 0.f ? rsqrtf(ss) : 0.f;
+  }
+  __syncthreads();
+  C[(int64_t)l * dp + f] = __float2bfloat16(acc * sinv);
 }
 
 // Key tiles of a query block: the tiles holding a row of a cell probed by one
@@ -248,31 +296,59 @@ __global__ void k_ivf_permute_probes(const int32_t* __restrict__ order, const in
 // the FP64 norms, rounded once to FP32), sorted by (cosine desc, original
 // index asc); the K best go to the row's original position with original
 // indices.
-__global__ void k_ivf_rerank(const float* __restrict__ X, int d, const double* __restrict__ nrm2,
-                             const int32_t* __restrict__ order, int64_t n, const float* __restrict__ cand_val,
-                             const int32_t* __restrict__ cand_idx, int K, int32_t* __restrict__ out_idx,
-                             float* __restrict__ out_sim) {
-  const int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+//
+// The candidates' rows are read 32 features at a time with coalesced loads
+// into shared memory, from which each lane takes its own row's values in
+// order (a lane reading its row from global memory cost a sector per
+// 4 bytes: 3.1 ms at n = 600,000, d = 100, 2.2 ms now, near what its 7.7 GB of
+// scattered rows take).
+constexpr int kIvfWarps = 8;
+constexpr int kIvfSeg = 32;  // features per step; rows of 33 floats keep the lanes on distinct banks
+__global__ void __launch_bounds__(kIvfWarps * 32)
+k_ivf_rerank(const float* __restrict__ X, int d, const double* __restrict__ nrm2, const int32_t* __restrict__ order,
+             int64_t n, const float* __restrict__ cand_val, const int32_t* __restrict__ cand_idx, int K,
+             int32_t* __restrict__ out_idx, float* __restrict__ out_sim) {
+  __shared__ float seg[kIvfWarps][32][kIvfSeg + 1];
+  const int64_t p = (int64_t)blockIdx.x * kIvfWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (p >= n) return;
+  float (*sg)[kIvfSeg + 1] = seg[threadIdx.x >> 5];
   const int64_t i = order[p];
   const int32_t jc = cand_idx[p * kCandC + lane];
   const int64_t j = jc >= 0 ? (int64_t)order[jc] : -1;
-  float s = -INFINITY;
-  if (j >= 0) {
-    const float* xi = X + i * d;
-    const float* xj = X + j * d;
-    // compensated dot product (Ogita, Rump and Oishi's Dot2: TwoProduct by
-    // FMA, TwoSum of the running sum), ~2^-44 relative before the division
-    float hi = 0.f, lo = 0.f;
-    for (int f = 0; f < d; ++f) {
-      const float pr = xi[f] * xj[f];
-      const float pe = fmaf(xi[f], xj[f], -pr);
+  const float* xi = X + i * d;
+  // compensated dot product (Ogita, Rump and Oishi's Dot2: TwoProduct by
+  // FMA, TwoSum of the running sum), ~2^-44 relative before the division
+  float hi = 0.f, lo = 0.f;
+  for (int f0 = 0; f0 < d; f0 += kIvfSeg) {
+    const int w = min(kIvfSeg, d - f0);
+    const bool in = lane < w;
+#pragma unroll
+    for (int r0 = 0; r0 < 32; r0 += 8) {
+      float v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int64_t jr = __shfl_sync(0xffffffffu, j, r0 + r);
+        v[r] = in && jr >= 0 ? X[jr * d + f0 + lane] : 0.f;
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) sg[r0 + r][lane] = v[r];
+    }
+    const float xv = in ? xi[f0 + lane] : 0.f;
+    __syncwarp();
+    for (int f = 0; f < w; ++f) {
+      const float a = __shfl_sync(0xffffffffu, xv, f), b = sg[lane][f];
+      const float pr = a * b;
+      const float pe = fmaf(a, b, -pr);
       const float t = hi + pr;
       const float z = t - hi;
       lo += (hi - (t - z)) + (pr - z) + pe;
       hi = t;
     }
+    __syncwarp();
+  }
+  float s = -INFINITY;
+  if (j >= 0) {
     const double ni = nrm2[i], nj = nrm2[j];
     s = (ni > 0.0 && nj > 0.0) ? (float)(((double)hi + (double)lo) / sqrt(ni * nj)) : 0.f;
   }
@@ -343,18 +419,20 @@ ancka_status exclusive_scan_i64(Workspace&, const int64_t* in, int64_t* out, int
 // = row, and the cells' offsets (nlist + 1)
 ancka_status sort_by_cell(Workspace& ws, const int32_t* cell, const int32_t* seq, int64_t n, int nlist, int32_t* order,
                           int64_t* cell_off, cudaStream_t s) {
-  const int64_t nchunks = ceil_div(n, kIvfChunk);
+  const int chunk = ivf_chunk(nlist);
+  const int64_t nchunks = ceil_div(n, chunk);
   int32_t* hist;
   int64_t* size;
   ANCKA_TRY(ws.zeros(&hist, (size_t)nchunks * nlist));
   ANCKA_TRY(ws.alloc(&size, (size_t)nlist));
-  k_ivf_hist<<<(unsigned)nchunks, 256, 0, s>>>(cell, seq, n, nlist, hist);
+  k_ivf_hist<<<(unsigned)nchunks, 256, 0, s>>>(cell, seq, n, nlist, chunk, hist);
   ANCKA_LAUNCHED();
-  k_ivf_cell_scan<<<grid_for(nlist, 128), 128, 0, s>>>(hist, nchunks, nlist, size);
+  k_ivf_cell_scan<<<grid_for(nlist, 4), 128, 0, s>>>(hist, nchunks, nlist, size);
   ANCKA_LAUNCHED();
   k_ivf_exscan<<<1, 1024, 0, s>>>(size, nlist, cell_off);
   ANCKA_LAUNCHED();
-  k_ivf_place<<<grid_for(nchunks, 64), 64, 0, s>>>(cell, seq, n, nlist, hist, cell_off, order);
+  // shared memory for nlist <= 8192 positions: 32 KB at most
+  k_ivf_place<<<(unsigned)nchunks, 32, sizeof(int32_t) * nlist, s>>>(cell, seq, n, nlist, chunk, hist, cell_off, order);
   ANCKA_LAUNCHED();
   return ANCKA_OK;
 }
@@ -401,7 +479,7 @@ ancka_status knn_ivf(Workspace& ws, const float* X, int64_t n, int32_t d, int32_
     ANCKA_TRY(sort_by_cell(ws, cell, nullptr, n_train, nlist, order, cell_off, s));
     k_ivf_map_order<<<grid_for(n_train, 256), 256, 0, s>>>(n_train < n ? train_rows : nullptr, n_train, order);
     ANCKA_LAUNCHED();
-    k_ivf_update<<<grid_for((int64_t)nlist * 32, 256), 256, 0, s>>>(pr.xb, dp, order, cell_off, nlist, C);
+    k_ivf_update<<<(unsigned)nlist, dp, 0, s>>>(pr.xb, dp, order, cell_off, nlist, C);  // dp <= 512
     ANCKA_LAUNCHED();
   }
   // 2. every row's nprobe nearest cells; its own cell is the first
@@ -463,7 +541,7 @@ ancka_status knn_ivf(Workspace& ws, const float* X, int64_t n, int32_t d, int32_
   ANCKA_TRY(knn_lists_bf16(ws, xs, pr.n_pad, nullptr, n, xs, n, pr.n_pad, dp, d, blk_ptr, blk_tiles, work, false, cv,
                            ci, terr, s));
   // 6. exact cosines of the candidates, back to the original order
-  k_ivf_rerank<<<grid_for(n * 32, 256), 256, 0, s>>>(X, d, pr.nrm2, order, n, cv, ci, K, out_idx, out_sim);
+  k_ivf_rerank<<<grid_for(n, kIvfWarps), kIvfWarps * 32, 0, s>>>(X, d, pr.nrm2, order, n, cv, ci, K, out_idx, out_sim);
   ANCKA_LAUNCHED();
   int32_t he = 0;
   ANCKA_CUDA(cudaMemcpyAsync(&he, terr, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
