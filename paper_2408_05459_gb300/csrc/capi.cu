@@ -226,8 +226,13 @@ ancka_status knn_impl(Workspace& ws, const float* X, int64_t n, int32_t d, int32
                       int32_t* idx, float* sim, int32_t** zero_row, int64_t* ncand, int64_t* nfb,
                       int64_t* nex, bool counts, cudaStream_t s, cudaEvent_t* contract_ev = nullptr,
                       const std::function<ancka_status()>& after_contraction = {}) {
+  // K beyond what two lists certify: the wide path, whatever the precision
+  // asked for (the lists are exact); it keeps the query block of the BF16
+  // contraction in shared memory.  An exhaustive FP32 scan of every pair, the
+  // route left for larger d, took 11.1 ms at n = 3001, d = 500, K = 50.
+  const bool wide = K > max_candidate_K(prec) && round_up(d, 64) <= knn_tc_max_dp();
   PrepOut pr;
-  ANCKA_TRY(prep_rows(ws, X, n, d, prec, &pr, s));
+  ANCKA_TRY(prep_rows(ws, X, n, d, wide ? ANCKA_PREC_BF16 : prec, &pr, s));
   if (zero_row) *zero_row = pr.zero_row;
   // the candidate lists certify K when a few slots of slack remain: one list
   // of 32 (CUDA-core contraction) or two of 16 (tensor-core contraction)
@@ -263,6 +268,17 @@ ancka_status knn_impl(Workspace& ws, const float* X, int64_t n, int32_t d, int32
                          prec == ANCKA_PREC_FP32 ? 1 : 2, prec == ANCKA_PREC_FP32 ? prec : ANCKA_PREC_BF16, terr, idx,
                          sim, ncand, nfb, nex, counts, s));
     if (contract_ev) ANCKA_CUDA(cudaEventRecord(contract_ev[2], s));
+  } else if (wide) {
+    ancka_status st;
+    {
+      Workspace wide_ws(s);  // ~1 KB a row and up to 2 GB of collected keys
+      st = knn_wide(wide_ws, X, n, d, K, pr, tc_acc_bound(pr.dp, 16, -22), idx, sim, nfb, nex, counts, s);
+    }
+    if (st == ANCKA_ERR_OOM)  // the exhaustive scan needs none of that
+      st = knn_rerank(ws, X, n, d, K, pr, ANCKA_PREC_FP32, 0.f, 0.f, nullptr, nullptr, 1, ANCKA_PREC_FP32, nullptr, idx,
+                      sim, ncand, nfb, nex, counts, s);
+    ANCKA_TRY(st);
+    if (after_contraction) ANCKA_TRY(after_contraction());
   } else {
     if (after_contraction) ANCKA_TRY(after_contraction());
     ANCKA_TRY(knn_rerank(ws, X, n, d, K, pr, ANCKA_PREC_FP32, 0.f, 0.f, nullptr, nullptr, 1, ANCKA_PREC_FP32,

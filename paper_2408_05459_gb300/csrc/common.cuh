@@ -213,6 +213,10 @@ ancka_status knn_candidates_bf16(Workspace& ws, const PrepOut& pr, int64_t n, fl
 ancka_status knn_candidates_fp8(Workspace& ws, const PrepOut& pr, int64_t n, float* cand_val, int32_t* cand_idx,
                                 int32_t* err, cudaStream_t s);
 int knn_tc_max_dp_fp8();
+// BF16 lists of every row against `shares` interleaved shares of the key
+// tiles: 2 x shares lists of 16 per row (n x shares x kCandC)
+ancka_status knn_candidates_bf16_shares(Workspace& ws, const PrepOut& pr, int64_t n, int shares, float* cand_val,
+                                        int32_t* cand_idx, int32_t* err, cudaStream_t s);
 // ivf.cu: approximate KNN by inverted lists (spherical k-means cells, nprobe
 // nearest cells per row, exact cosines of the candidates found there)
 struct IvfStats {
@@ -267,6 +271,13 @@ ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int
                         int32_t* cand_idx, int lists, int collect_prec, const int32_t* list_err, int32_t* out_idx,
                         float* out_sim, int64_t* n_candidates, int64_t* n_fallback, int64_t* n_exhaustive,
                         bool want_counts, cudaStream_t s);
+
+// rerank.cu: exact lists for K up to 64 from 2 x shares lists and the collect
+// pass (BF16 copy in pr, pr.dp <= knn_tc_max_dp()); reads nothing back unless
+// want_counts
+ancka_status knn_wide(Workspace& ws, const float* X, int64_t n, int32_t d, int32_t K, const PrepOut& pr, float acc,
+                      int32_t* out_idx, float* out_sim, int64_t* n_fallback, int64_t* n_exhaustive, bool want_counts,
+                      cudaStream_t s);
 
 // graph.cu: walk structures
 struct Csr {

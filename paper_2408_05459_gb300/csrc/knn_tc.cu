@@ -692,13 +692,16 @@ __device__ __forceinline__ void pair_arrive(uint32_t bar) {
 }
 
 // One CTA of the pair; grid = 2 x pairs.  Arguments as for k_knn_tc; part_*
-// hold two slots of kPairRows rows per pair.
+// hold two slots of kPairRows rows per pair.  With shares > 1 each block of
+// rows is swept once per share of the key tiles (tiles share, share + shares,
+// ...; past the last one the keys are padding), and row i leaves two lists per
+// share, at (i * shares + share) * kCandC; qblocks counts (block, share) pairs.
 template <bool kE4M3>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
            int64_t n_pad, int64_t qblocks, int kb_count, int k_last, int nstages, float* __restrict__ cand_val,
            int32_t* __restrict__ cand_idx, const float* __restrict__ out_scale, float* __restrict__ part_val,
-           int32_t* __restrict__ part_idx, const int32_t* __restrict__ a_rows, int64_t n_rows,
+           int32_t* __restrict__ part_idx, const int32_t* __restrict__ a_rows, int64_t n_rows, int shares,
            unsigned long long* __restrict__ tick, int* __restrict__ err) {
   constexpr int kTK = kE4M3 ? 128 : 64;  // features per stage
   extern __shared__ uint8_t smem_raw[];
@@ -710,7 +713,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int64_t pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
-  const int n_tiles = (int)ceil_div(n_pad, kTN);
+  const int n_tiles = (int)ceil_div(ceil_div(n_pad, kTN), shares);
   const int64_t work = qblocks * n_tiles;
   const int64_t w_begin = range_begin(pair, work, pairs);
   const int64_t w_end = range_begin(pair + 1, work, pairs);
@@ -759,6 +762,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
       for (int64_t w = w_begin; w < w_end && ok; ++seg) {
         const Seg sg = segment_at(w, w_end, n_tiles, qblocks, none);
+        const int share = (int)(sg.qb % shares);
         w += sg.t1 - sg.t0;
         // the previous query rows stay in use until their last MMA completes
         if (seg > 0 && !mbar_wait_warp(&bars->a_empty, (uint32_t)((seg - 1) & 1), abort, err, 6)) {
@@ -794,11 +798,11 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         if (elect_one()) {
           if (leader) mbar_expect_tx(&bars->a_full, (uint32_t)(2 * kb_count * kABytes));
           for (int kb = 0; kb < kb_count; ++kb)
-            pair_tma_load(sA0 + kb * kABytes, &tmA, kb * kTK, (int)(sg.qb * kPairRows + rank * kTM), a_full);
+            pair_tma_load(sA0 + kb * kABytes, &tmA, kb * kTK, (int)(sg.qb / shares * kPairRows + rank * kTM), a_full);
         }
         __syncwarp();
         for (int t = sg.t0; t < sg.t1 && ok; ++t) {
-          const int kt = t + rot < n_tiles ? t + rot : t + rot - n_tiles;
+          const int kt = (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * shares + share;
           for (int kb = 0; kb < kb_count; ++kb) {
             if (!mbar_wait_warp(&bars->empty[stage], phase ^ 1, abort, err, 1)) {
               ok = false;
@@ -899,9 +903,10 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
     bool ok = true;
     for (int64_t w = w_begin; w < w_end && ok; ++seg) {
       const Seg sg = segment_at(w, w_end, n_tiles, qblocks, none);
+      const int share = (int)(sg.qb % shares);
       int rot = 0;
       w += sg.t1 - sg.t0;
-      const int64_t ra = sg.qb * kPairRows + rank * kTM + r;
+      const int64_t ra = sg.qb / shares * kPairRows + rank * kTM + r;
       const bool row_ok = ra < n_rows;
       const int64_t i = a_rows ? (row_ok ? (int64_t)a_rows[ra] : -1) : ra;
       RowList<C> L;
@@ -917,7 +922,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         // written before the segment's query rows were loaded, which its
         // first accumulator waited for
         if (t == sg.t0) rot = *reinterpret_cast<volatile int*>(&bars->rot[seg & 1]);
-        const int kt = t + rot < n_tiles ? t + rot : t + rot - n_tiles;
+        const int kt = (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * shares + share;
         const uint32_t jb = (uint32_t)kt * kTN + (uint32_t)(h * kSliceN);
         const uint32_t tb = lane_base + (uint32_t)(b * kTN);
         auto release = [&] {
@@ -933,8 +938,8 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       int32_t* oi;
       if (sg.t0 == 0 && sg.t1 == n_tiles) {  // whole block: final lists
         if (!row_ok) continue;
-        ov = cand_val + i * kCandC;
-        oi = cand_idx + i * kCandC;
+        ov = cand_val + (i * shares + share) * kCandC;
+        oi = cand_idx + (i * shares + share) * kCandC;
       } else {
         const int64_t slot = (pair * 2 + (seg == 0 ? 0 : 1)) * kPairRows + rank * kTM + r;
         ov = part_val + slot * kCandC;
@@ -970,16 +975,16 @@ template <int kRows>
 __global__ void __launch_bounds__(2 * kRows)
 k_merge_lists(int n_tiles, int64_t work, int64_t ctas, const int64_t* __restrict__ blk_ptr,
               const float* __restrict__ part_val, const int32_t* __restrict__ part_idx,
-              const int32_t* __restrict__ a_rows, int64_t n_rows, float* __restrict__ cand_val,
+              const int32_t* __restrict__ a_rows, int64_t n_rows, int shares, float* __restrict__ cand_val,
               int32_t* __restrict__ cand_idx) {
   static_assert(kLists == 2 && kListC == 16, "a thread per half, four 16-byte loads per list");
   const int64_t qb = blockIdx.x;
   const int64_t x0 = blk_ptr ? blk_ptr[qb] : qb * n_tiles;
   const int64_t x1 = blk_ptr ? blk_ptr[qb + 1] : x0 + n_tiles;
   const int r = threadIdx.x % kRows, h = threadIdx.x / kRows;
-  const int64_t ra = qb * kRows + r;
+  const int64_t ra = qb / shares * kRows + r;
   if (ra >= n_rows) return;
-  const int64_t i = a_rows ? (int64_t)a_rows[ra] : ra;
+  const int64_t i = (a_rows ? (int64_t)a_rows[ra] : ra) * shares + qb % shares;  // the lists' row
   constexpr int C = kListC;
   float* ov = cand_val + i * kCandC + h * C;
   int32_t* oi = cand_idx + i * kCandC + h * C;
@@ -1502,7 +1507,7 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
   ANCKA_LAUNCHED();
   if (!kCollect) {
     k_merge_lists<kTM><<<(unsigned)qblocks, 2 * kTM, 0, s>>>(n_tiles, work, ctas, ca.blk_ptr, part_val, part_idx, ca.a_rows,
-                                                    n_rows, cand_val, cand_idx);
+                                                    n_rows, 1, cand_val, cand_idx);
     ANCKA_LAUNCHED();
   }
   return ANCKA_OK;
@@ -1513,7 +1518,7 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
 template <bool kE4M3>
 ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& tb, int64_t n, int64_t n_pad,
                          const int32_t* a_rows, int64_t n_rows, int kb_count, int d, float* cand_val,
-                         int32_t* cand_idx, const float* out_scale, int32_t* err, cudaStream_t s) {
+                         int32_t* cand_idx, const float* out_scale, int32_t* err, cudaStream_t s, int shares = 1) {
   const int per_kb = kE4M3 ? 128 : 64, per_mma = kE4M3 ? 32 : 16;  // k_last as in launch_tc
   const int rem = d - per_kb * (kb_count - 1);
   const int k_last = (rem >= 1 && rem <= per_kb) ? (int)ceil_div(rem, per_mma) : kMmaPerStage;
@@ -1527,8 +1532,8 @@ ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap
   int sms = 152, dev = 0;
   ANCKA_CUDA(cudaGetDevice(&dev));
   ANCKA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t qblocks = ceil_div(n_rows, kPairRows);
-  const int n_tiles = (int)ceil_div(n_pad, kTN);
+  const int64_t qblocks = ceil_div(n_rows, kPairRows) * shares;
+  const int n_tiles = (int)ceil_div(ceil_div(n_pad, kTN), shares);
   const int64_t work = qblocks * n_tiles;
   const int64_t pairs = std::max<int64_t>(1, std::min<int64_t>(sms / 2, work));
   float* part_val;
@@ -1540,10 +1545,10 @@ ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap
   ANCKA_CUDA(cudaFuncSetAttribute(k_knn_pair<kE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k_knn_pair<kE4M3><<<(unsigned)(2 * pairs), kPairThreads, smem, s>>>(
       ta, tb, n, n_pad, qblocks, kb_count, k_last, nstages, cand_val, cand_idx, out_scale, part_val, part_idx,
-      a_rows, n_rows, tick, err);
+      a_rows, n_rows, shares, tick, err);
   ANCKA_LAUNCHED();
   k_merge_lists<kPairRows><<<(unsigned)qblocks, 2 * kPairRows, 0, s>>>(n_tiles, work, pairs, nullptr, part_val, part_idx,
-                                                                   a_rows, n_rows, cand_val, cand_idx);
+                                                                   a_rows, n_rows, shares, cand_val, cand_idx);
   ANCKA_LAUNCHED();
   return ANCKA_OK;
 }
@@ -1637,6 +1642,16 @@ ancka_status knn_candidates_bf16(Workspace& ws, const PrepOut& pr, int64_t n, fl
   }
   ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN / 2, 2));
   return launch_pair<false>(ws, ta, tb, n, pr.n_pad, nullptr, n, kb_count, pr.d, cand_val, cand_idx, nullptr, err, s);
+}
+
+// two lists per row and share of the key tiles (see k_knn_pair)
+ancka_status knn_candidates_bf16_shares(Workspace& ws, const PrepOut& pr, int64_t n, int shares, float* cand_val,
+                                        int32_t* cand_idx, int32_t* err, cudaStream_t s) {
+  CUtensorMap ta, tb;
+  ANCKA_TRY(make_map(&ta, pr.xb, pr.dp, pr.n_pad, kTM, 2));
+  ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN / 2, 2));
+  return launch_pair<false>(ws, ta, tb, n, pr.n_pad, nullptr, n, pr.dp / 64, pr.d, cand_val, cand_idx, nullptr, err, s,
+                            shares);
 }
 
 void knn_set_symmetric_min_rows(int64_t n_min) { g_sym_min_rows.store(n_min, std::memory_order_relaxed); }

@@ -622,6 +622,136 @@ __global__ void k_exh_merge(const int32_t* __restrict__ rows, const int32_t* __r
   }
 }
 
+
+// ---------------------------------------------------------------------------
+// K beyond what two 16-entry lists certify (up to 64).  The sweep leaves
+// 2 x shares lists a row, each over its own share of the keys; the K-th
+// largest lower bound among their entries bounds the true K-th similarity
+// from below, whichever keys the lists missed.  The collect pass then gathers
+// every key that can still reach it, and those are scored exactly.
+// ---------------------------------------------------------------------------
+
+// thr[i] = (K-th largest lower bound of row i's per candidates) - m_max, or
+// -inf when there are fewer than K (every key is collected); one warp per row
+__global__ void __launch_bounds__(kWarps * 32)
+k_wide_threshold(const float* __restrict__ cand_val, const int32_t* __restrict__ cand_idx, int per, int64_t n, int K,
+                 const float* __restrict__ err, const float* __restrict__ err_max_p, float acc,
+                 int32_t* __restrict__ rows, float* __restrict__ thr) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (i >= n) return;
+  const float ei = err[i], emax = *err_max_p;
+  uint32_t key[4];  // 0: no candidate (below every number's key)
+  int nvalid = 0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int e = u * 32 + lane;
+    const int32_t j = e < per ? cand_idx[i * per + e] : -1;
+    key[u] = 0;
+    if (j >= 0) {
+      const float ej = err[j];
+      key[u] = fkey(cand_val[i * per + e] - (ei * (1.f + ej) + ej + acc * (1.f + ei) * (1.f + ej)));
+    }
+    nvalid += __popc(__ballot_sync(0xffffffffu, j >= 0));
+  }
+  uint32_t kth = 0;  // the largest key that at least K candidates reach
+  for (int b = 31; b >= 0; --b) {
+    const uint32_t t = kth | (1u << b);
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) c += __popc(__ballot_sync(0xffffffffu, key[u] >= t));
+    if (c >= K) kth = t;
+  }
+  if (lane == 0) {
+    const float mmax = ei * (1.f + emax) + emax + acc * (1.f + ei) * (1.f + emax);
+    rows[i] = (int32_t)i;
+    thr[i] = nvalid >= K ? fkey_value(kth) - mmax : -INFINITY;
+  }
+}
+
+// The K best of the keys collected for rows row0 .. row0 + count - 1, one CTA
+// per row: four candidates a warp at a time into shared memory as Dot2 pairs,
+// then the exhaustive kernels' FP64 cosines (one candidate a lane, so the
+// narrow FP64 pipe sees 32 of them per instruction) and a bitonic sort by
+// (cosine desc, index asc).  The sums and cosines have the bits of the
+// exhaustive kernels.  A row whose buffer overflowed or holds fewer than K
+// keys, and every row after a failed pass, goes to the exhaustive kernels.
+constexpr int kWideCap = 2048;
+constexpr int kWideWarps = 4;
+__global__ void __launch_bounds__(kWideWarps * 32)
+k_rerank_wide(const float* __restrict__ X, int d, int K, const double* __restrict__ rinv, int64_t row0, int64_t count,
+              const int32_t* __restrict__ cnt, const int32_t* __restrict__ buf, int32_t* __restrict__ out_idx,
+              float* __restrict__ out_sim, int32_t* __restrict__ ov_rows, int32_t* __restrict__ ov_count,
+              const int32_t* __restrict__ list_err, const int32_t* __restrict__ collect_err) {
+  __shared__ unsigned long long sk[kWideCap];
+  __shared__ int32_t si[kWideCap];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t r = blockIdx.x;
+  const int64_t i = row0 + r;
+  const int c = cnt[r];
+  if (c > kWideCap || c < K || *list_err || *collect_err) {
+    if (threadIdx.x == 0) ov_rows[atomicAdd(ov_count, 1)] = (int32_t)i;
+    return;
+  }
+  const float* xi = X + i * (int64_t)d;
+  const int32_t* keys = buf + r * kWideCap;
+  SparseRow sp;
+  sparse_row(xi, d, sp);
+  const bool sparse = sp.cmax <= kSpLane && sp.cmax < (d + 31) / 32;  // warp-uniform
+  for (int b = warp * 4; b < c; b += kWideWarps * 4) {
+    int32_t jt[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) jt[u] = b + u < c ? keys[b + u] : -1;
+    float ds[4], dc[4];
+    if (sparse)
+      dot2_sparse4(X, d, sp, jt, ds, dc);
+    else
+      dot2_rows4(X, xi, d, jt, ds, dc);
+    float rs, rc;
+    dot2_reduce4(ds, dc, rs, rc);  // lane 8u holds partial u
+    const int u = lane >> 3;
+    if ((lane & 7) == 0 && b + u < c) {
+      sk[b + u] = ((unsigned long long)__float_as_uint(rs) << 32) | __float_as_uint(rc);
+      si[b + u] = u == 0 ? jt[0] : u == 1 ? jt[1] : u == 2 ? jt[2] : jt[3];
+    }
+  }
+  __syncthreads();
+  int p = 2;
+  while (p < c) p <<= 1;
+  const double ri = rinv[i];
+  for (int e = threadIdx.x; e < p; e += blockDim.x) {
+    if (e < c) {
+      const unsigned long long v = sk[e];
+      sk[e] = dkey(cos_from(__uint_as_float((uint32_t)(v >> 32)), __uint_as_float((uint32_t)v), ri, rinv[si[e]]));
+    } else {
+      sk[e] = 0;
+      si[e] = INT32_MAX;
+    }
+  }
+  for (int k = 2; k <= p; k <<= 1)
+    for (int s = k >> 1; s > 0; s >>= 1) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < p / 2; e += blockDim.x) {
+        const int a = 2 * e - (e & (s - 1));  // the e-th index whose bit s is clear
+        const int b = a + s;
+        const unsigned long long ka = sk[a], kb = sk[b];
+        const int32_t ja = si[a], jb = si[b];
+        const bool a_first = ka > kb || (ka == kb && ja < jb);
+        if (a_first != ((a & k) == 0)) {
+          sk[a] = kb;
+          sk[b] = ka;
+          si[a] = jb;
+          si[b] = ja;
+        }
+      }
+    }
+  __syncthreads();
+  for (int e = threadIdx.x; e < K; e += blockDim.x) {
+    out_idx[i * K + e] = si[e];
+    out_sim[i * K + e] = (float)dkey_value(sk[e]);
+  }
+}
+
 }  // namespace
 
 ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int32_t K,
@@ -752,6 +882,68 @@ ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int
       *n_candidates = (int64_t)nc;
       if (ex_count_dev && n_exhaustive) *n_exhaustive = ex;
     }
+  }
+  return ANCKA_OK;
+}
+
+// Exact lists of K > the lists' certificate.  No host read: a failed pass
+// sends its rows to the exhaustive kernels on the device.
+ancka_status knn_wide(Workspace& ws, const float* X, int64_t n, int32_t d, int32_t K, const PrepOut& pr, float acc,
+                      int32_t* out_idx, float* out_sim, int64_t* n_fallback, int64_t* n_exhaustive, bool want_counts,
+                      cudaStream_t s) {
+  // a list of 16 holds its share of the K best with room to spare (K = 64:
+  // 8 of 16 on average); a miss only lowers the threshold
+  const int shares = K <= 15 ? 1 : (K <= 31 ? 2 : 4);
+  const int per = shares * kCandC;
+  double* rinv;
+  float2* rinv2;
+  float *cv, *thr;
+  int32_t *ci, *rows, *cnt, *buf, *ov_rows, *ov_count, *errs;
+  ANCKA_TRY(ws.alloc(&rinv, (size_t)n));
+  ANCKA_TRY(ws.alloc(&rinv2, (size_t)n));
+  ANCKA_TRY(ws.alloc(&cv, (size_t)n * per));
+  ANCKA_TRY(ws.alloc(&ci, (size_t)n * per));
+  ANCKA_TRY(ws.alloc(&thr, (size_t)n));
+  ANCKA_TRY(ws.alloc(&rows, (size_t)n));
+  ANCKA_TRY(ws.alloc(&ov_rows, (size_t)n));
+  ANCKA_TRY(ws.zeros(&ov_count, 1));
+  ANCKA_TRY(ws.zeros(&errs, 2));  // list pass, collect pass
+  k_inv_norms<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(pr.nrm2, n, rinv, rinv2);
+  ANCKA_LAUNCHED();
+  ANCKA_TRY(knn_candidates_bf16_shares(ws, pr, n, shares, cv, ci, errs, s));
+  k_wide_threshold<<<(unsigned)ceil_div(n, kWarps), kWarps * 32, 0, s>>>(cv, ci, per, n, K, pr.err, pr.err_max, acc,
+                                                                         rows, thr);
+  ANCKA_LAUNCHED();
+  // the collected keys of kChunk rows at a time: 2 GB of buffer at most
+  constexpr int64_t kChunk = 1 << 18;
+  const int64_t chunk = n < kChunk ? n : kChunk;
+  ANCKA_TRY(ws.alloc(&cnt, (size_t)chunk));
+  ANCKA_TRY(ws.alloc(&buf, (size_t)chunk * kWideCap));
+  for (int64_t r0 = 0; r0 < n; r0 += chunk) {
+    const int64_t m = n - r0 < chunk ? n - r0 : chunk;
+    Workspace pass(s);
+    ANCKA_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * m, s));
+    ANCKA_TRY(knn_collect_bf16(pass, pr, n, rows + r0, m, thr + r0, cnt, buf, kWideCap, errs + 1, s));
+    k_rerank_wide<<<(unsigned)m, kWideWarps * 32, 0, s>>>(X, d, K, rinv, r0, m, cnt, buf, out_idx, out_sim, ov_rows,
+                                                          ov_count, errs, errs + 1);
+    ANCKA_LAUNCHED();
+  }
+  double* pv;
+  int32_t* pi;
+  ANCKA_TRY(ws.alloc(&pv, (size_t)kSlicedMaxRows * kSlices * K));
+  ANCKA_TRY(ws.alloc(&pi, (size_t)kSlicedMaxRows * kSlices * K));
+  k_exh_sliced<<<1216, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ov_rows, ov_count, pv, pi);
+  ANCKA_LAUNCHED();
+  k_exh_merge<<<8, 128, 0, s>>>(ov_rows, ov_count, K, pv, pi, out_idx, out_sim);
+  ANCKA_LAUNCHED();
+  k_knn_exhaustive<<<304, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ov_rows, ov_count, 0, out_idx, out_sim);
+  ANCKA_LAUNCHED();
+  if (want_counts) {
+    int32_t ex = 0;
+    ANCKA_CUDA(cudaMemcpyAsync(&ex, ov_count, sizeof(ex), cudaMemcpyDeviceToHost, s));
+    ANCKA_CUDA(cudaStreamSynchronize(s));
+    *n_fallback = n;
+    if (n_exhaustive) *n_exhaustive = ex;
   }
   return ANCKA_OK;
 }
