@@ -12,12 +12,12 @@
 //              128 bytes of features per stage: 64 BF16 or 128 FP8) through
 //              an nstages-deep ring (mbarrier full/empty);
 //   warp 1     MMA issuer: allocates 512 TMEM columns, issues
-//              tcgen05.mma.cta_group::1.kind::f16 (BF16, K=16) or
-//              kind::f8f6f4 (E4M3, K=32) with M=128, N=256 into two
+//              tcgen05.mma.cta_group::1.kind::f16 (BF16, K=16) with M=128,
+//              N=256 (the pair: also kind::f8f6f4, E4M3, K=32) into two
 //              ping-pong FP32 accumulators, commits stage releases,
 //              accumulator-ready signals and the release of A at the end of
 //              each query block;
-//   warps 2-9  epilogue: two warps per TMEM lane quarter, each owning half of
+//   warps 4-11 epilogue: two warps per TMEM lane quarter, each owning half of
 //              every tile's 256 columns; tcgen05.ld (32x32b) of the thread's
 //              accumulator row (TMEM lane = query row), threshold test and
 //              insert into a register-resident list of its 16 best scores.
@@ -49,6 +49,14 @@ constexpr int kLists = 2;                // lists per row = column slices of eve
 constexpr int kEpiWarps = 4 * kLists;    // one warp per (TMEM lane quarter, column slice)
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kListC = kCandC / kLists;  // entries of each list
+// Three warpgroups: the producer, the MMA issuer and two idle warps, then the
+// eight epilogue warps.  What decides whether the MMAs wait is how soon an
+// accumulator comes back, so the epilogue takes all 128 columns of its slice
+// into registers before it looks at them; the first warpgroup gives up its
+// registers for that (setmaxnreg: 128 x 64 + 256 x 216 = 63,488 of the
+// 384 x 168 = 64,512 the block is launched with).
+constexpr int kTcThreads = 128 + 32 * kEpiWarps;
+constexpr int kRegsLow = 64, kRegsHigh = 216;
 constexpr int kSliceN = kTN / kLists;    // columns of a tile per slice
 constexpr int kABytes = kTM * kTKB;      // 16 KB per 128-byte block of A
 constexpr int kBBytes = kTN * kTKB;      // 32 KB per stage of B
@@ -82,13 +90,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
           tmem_d),
       "l"(da), "l"(db), "r"(kIdescBF16), "r"(accum)
-      : "memory");
-}
-__device__ __forceinline__ void umma_e4m3(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}" ::"r"(
-          tmem_d),
-      "l"(da), "l"(db), "r"(kIdescE4M3), "r"(accum)
       : "memory");
 }
 // Row lists are kept sorted in descending score order, lv[0] >= ... >=
@@ -211,37 +212,34 @@ __device__ __forceinline__ void collect_chunk(const uint32_t (&r)[32], float mx,
 }
 
 // Fold one tile's column slice (kSliceN accumulator columns from TMEM address
-// tb, keys jb ...) into the row's list, 64 columns at a time (all 128 would
-// not fit the registers of 10 warps): four 16-column loads with the
-// hardware's maximum of each behind one wait, then four independent votes
-// that say which chunks hold a key above some lane's threshold (two of the
-// tile's eight at n = 600,000).  release() hands the accumulator back once
-// the last column has landed, before the list work on it.
-template <int C, int kPart, class Release>
+// tb, keys jb ...) into the row's list: eight 16-column loads with the
+// hardware's maximum of each behind one wait, release() to hand the
+// accumulator back before any list work, then eight independent votes that say
+// which chunks hold a key above some lane's threshold (about one a tile at
+// n = 600,000).
+template <int C, class Release>
 __device__ __forceinline__ void fold_slice(uint32_t tb, uint32_t jb, uint32_t n, uint32_t i, RowList<C>& L,
                                            Release&& release) {
-#pragma unroll 1
-  for (int p = 0; p < kSliceN; p += 16 * kPart) {
-    uint32_t r[kPart][16];
-    float mx[kPart];
+  constexpr int kChunks = kSliceN / 16;
+  uint32_t r[kChunks][16];
+  float mx[kChunks];
 #pragma unroll
-    for (int c = 0; c < kPart; ++c) tmem_ld16_max_issue(tb + (uint32_t)(p + c * 16), r[c], mx[c]);
-    tmem_wait();
+  for (int c = 0; c < kChunks; ++c) tmem_ld16_max_issue(tb + (uint32_t)(c * 16), r[c], mx[c]);
+  tmem_wait();
 #pragma unroll
-    for (int c = 0; c < kPart; ++c) {
-      pin(r[c]);
-      pin1(mx[c]);
-    }
-    if (p + 16 * kPart == kSliceN) release();
-    const float thr = L.lv[C - 1];
-    uint32_t hit = 0;
-#pragma unroll
-    for (int c = 0; c < kPart; ++c) hit |= (__any_sync(0xffffffffu, mx[c] > thr) ? 1u : 0u) << c;
-    if (hit == 0) continue;
-#pragma unroll
-    for (int c = 0; c < kPart; ++c)
-      if (hit & (1u << c)) L.push(r[c], mx[c], jb + (uint32_t)(p + c * 16), n, i);
+  for (int c = 0; c < kChunks; ++c) {
+    pin(r[c]);
+    pin1(mx[c]);
   }
+  release();
+  const float thr = L.lv[C - 1];
+  uint32_t hit = 0;
+#pragma unroll
+  for (int c = 0; c < kChunks; ++c) hit |= (__any_sync(0xffffffffu, mx[c] > thr) ? 1u : 0u) << c;
+  if (hit == 0) return;
+#pragma unroll
+  for (int c = 0; c < kChunks; ++c)
+    if (hit & (1u << c)) L.push(r[c], mx[c], jb + (uint32_t)(c * 16), n, i);
 }
 
 struct CollectArgs {
@@ -310,21 +308,21 @@ __device__ __forceinline__ int key_rotation(int64_t qb, int n_tiles, int64_t wor
 }
 
 // kCollect: collect mode (keys above a per-row threshold) instead of list
-// mode (two 16-entry lists per row); kE4M3: FP8 operands.  out_scale (list
+// mode (two 16-entry lists per row).  out_scale (list
 // mode, may be null) multiplies the scores written out.
 // key_stride > 1: only every key_stride-th key tile is swept (the sampled
 // pass of the symmetric contraction).  k_last: MMAs issued for the last
 // 128-byte block of features (those past the last one holding a feature of
 // X are zero padding and are skipped).
-template <bool kCollect, bool kE4M3>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kCollect>
+__global__ void __launch_bounds__(kTcThreads, 1)
 k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
          int64_t n_pad, int64_t qblocks, int kb_count, int k_last, int nstages, int key_stride,
          float* __restrict__ cand_val,
          int32_t* __restrict__ cand_idx, const float* __restrict__ out_scale, float* __restrict__ part_val,
          int32_t* __restrict__ part_idx, CollectArgs ca, unsigned long long* __restrict__ tick,
          int* __restrict__ err) {
-  constexpr int kTK = kE4M3 ? 128 : 64;  // features per stage
+  constexpr int kTK = 64;  // features per stage
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -364,137 +362,136 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
 
-  if (warp == 0) {
-    bool pending[kMaxStages];
-    uint32_t pend_par[kMaxStages];
-    for (int s = 0; s < kMaxStages; ++s) pending[s] = false;
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    int seg = 0;
-    uint32_t tiles_issued = 0;
-    const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
-    for (int64_t w = w_begin; w < w_end && ok; ++seg) {
-      const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
-      const int64_t qb = sg.qb;
-      const int t0 = sg.t0, t1 = sg.t1;
-      int rot = ca.blk_ptr ? 0 : key_rotation(qb, n_tiles, work, gridDim.x);
-      w += t1 - t0;
-      // the previous block of A stays in use until its last MMA completes
-      if (seg > 0 && !mbar_wait_warp(&bars->a_empty, (uint32_t)((seg - 1) & 1), abort, err, 6)) {
-        ok = false;
-        break;
-      }
-      // A block this CTA sweeps whole starts at the key tile the CTAs are
-      // reading now (tiles issued by all CTAs / CTAs), so that CTAs whose
-      // rates drift apart re-align at every block and keep sharing the key
-      // tiles in L2; a split block keeps the static rotation both of its
-      // CTAs can compute.
-      if (tick && !ca.blk_ptr && t0 == 0 && t1 == n_tiles)
-        rot = (int)((*reinterpret_cast<volatile unsigned long long*>(tick) / gridDim.x) % (uint64_t)n_tiles);
-      rot = __shfl_sync(0xffffffffu, rot, 0);
-      if (elect_one()) {
-        bars->rot[seg & 1] = rot;
-        __threadfence_block();
-        mbar_expect_tx(&bars->a_full, (uint32_t)(kb_count * kABytes));
-        for (int kb = 0; kb < kb_count; ++kb)
-          tma_load_2d(sA0 + kb * kABytes, &tmA, kb * kTK, (int)(qb * kTM), &bars->a_full);
-      }
-      __syncwarp();
-      for (int t = t0; t < t1 && ok; ++t) {
-        const int kt = ca.blk_ptr ? ca.blk_tiles[sg.base + t]
-                                  : (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * key_stride;
-        for (int kb = 0; kb < kb_count; ++kb) {
-          if (!mbar_wait_warp(&bars->empty[stage], phase ^ 1, abort, err, 1)) {
-            ok = false;
-            break;
-          }
-          if (elect_one()) {
-            mbar_expect_tx(&bars->full[stage], (uint32_t)kBBytes);
-            tma_load_2d(sB0 + stage * kBBytes, &tmB, kb * kTK, kt * kTN, &bars->full[stage]);
-          }
-          __syncwarp();
-          pending[stage] = true;
-          pend_par[stage] = phase;
-          if (++stage == nstages) {
-            stage = 0;
-            phase ^= 1;
-          }
-        }
-        if (tick && ((++tiles_issued) & 15) == 0 && lane == 0) atomicAdd(tick, 16ull);
-      }
-    }
-    if (!ok) {  // drain this warp's copies still in flight (bounded)
-      if (seg > 0) mbar_wait(&bars->a_full, (uint32_t)((seg - 1) & 1), nullptr, nullptr, 0);
-      for (int s = 0; s < nstages; ++s)
-        if (pending[s]) mbar_wait(&bars->full[s], pend_par[s], nullptr, nullptr, 0);
-    }
-  } else if (warp == 1) {
-    bool ok = true;
-    int stage = 0;
-    uint32_t phase = 0;
-    bool issued = false;
-    int64_t g = 0;  // accumulator tiles so far (ping-pong over two)
-    int seg = 0;
-    const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
-    for (int64_t w = w_begin; w < w_end && ok; ++seg) {
-      const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
-      const int t0 = sg.t0, t1 = sg.t1;
-      w += t1 - t0;
-      if (!mbar_wait_warp(&bars->a_full, (uint32_t)(seg & 1), abort, err, 2)) {
-        ok = false;
-        break;
-      }
-      for (int t = t0; t < t1; ++t, ++g) {
-        const int b = (int)(g & 1);
-        const uint32_t use = (uint32_t)(g >> 1);
-        if (!mbar_wait_warp(&bars->tempty[b], (use & 1) ^ 1, abort, err, 3)) {
+  if (warp < 4) {
+    if constexpr (!kCollect) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
+    if (warp == 0) {
+      bool pending[kMaxStages];
+      uint32_t pend_par[kMaxStages];
+      for (int s = 0; s < kMaxStages; ++s) pending[s] = false;
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      int seg = 0;
+      uint32_t tiles_issued = 0;
+      const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+      for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+        const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
+        const int64_t qb = sg.qb;
+        const int t0 = sg.t0, t1 = sg.t1;
+        int rot = ca.blk_ptr ? 0 : key_rotation(qb, n_tiles, work, gridDim.x);
+        w += t1 - t0;
+        // the previous block of A stays in use until its last MMA completes
+        if (seg > 0 && !mbar_wait_warp(&bars->a_empty, (uint32_t)((seg - 1) & 1), abort, err, 6)) {
           ok = false;
           break;
         }
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(b * kTN);
-        for (int kb = 0; kb < kb_count; ++kb) {
-          if (!mbar_wait_warp(&bars->full[stage], phase, abort, err, 4)) {
+        // A block this CTA sweeps whole starts at the key tile the CTAs are
+        // reading now (tiles issued by all CTAs / CTAs), so that CTAs whose
+        // rates drift apart re-align at every block and keep sharing the key
+        // tiles in L2; a split block keeps the static rotation both of its
+        // CTAs can compute.
+        if (tick && !ca.blk_ptr && t0 == 0 && t1 == n_tiles)
+          rot = (int)((*reinterpret_cast<volatile unsigned long long*>(tick) / gridDim.x) % (uint64_t)n_tiles);
+        rot = __shfl_sync(0xffffffffu, rot, 0);
+        if (elect_one()) {
+          bars->rot[seg & 1] = rot;
+          __threadfence_block();
+          mbar_expect_tx(&bars->a_full, (uint32_t)(kb_count * kABytes));
+          for (int kb = 0; kb < kb_count; ++kb)
+            tma_load_2d(sA0 + kb * kABytes, &tmA, kb * kTK, (int)(qb * kTM), &bars->a_full);
+        }
+        __syncwarp();
+        for (int t = t0; t < t1 && ok; ++t) {
+          const int kt = ca.blk_ptr ? ca.blk_tiles[sg.base + t]
+                                    : (t + rot < n_tiles ? t + rot : t + rot - n_tiles) * key_stride;
+          for (int kb = 0; kb < kb_count; ++kb) {
+            if (!mbar_wait_warp(&bars->empty[stage], phase ^ 1, abort, err, 1)) {
+              ok = false;
+              break;
+            }
+            if (elect_one()) {
+              mbar_expect_tx(&bars->full[stage], (uint32_t)kBBytes);
+              tma_load_2d(sB0 + stage * kBBytes, &tmB, kb * kTK, kt * kTN, &bars->full[stage]);
+            }
+            __syncwarp();
+            pending[stage] = true;
+            pend_par[stage] = phase;
+            if (++stage == nstages) {
+              stage = 0;
+              phase ^= 1;
+            }
+          }
+          if (tick && ((++tiles_issued) & 15) == 0 && lane == 0) atomicAdd(tick, 16ull);
+        }
+      }
+      if (!ok) {  // drain this warp's copies still in flight (bounded)
+        if (seg > 0) mbar_wait(&bars->a_full, (uint32_t)((seg - 1) & 1), nullptr, nullptr, 0);
+        for (int s = 0; s < nstages; ++s)
+          if (pending[s]) mbar_wait(&bars->full[s], pend_par[s], nullptr, nullptr, 0);
+      }
+    } else if (warp == 1) {
+      bool ok = true;
+      int stage = 0;
+      uint32_t phase = 0;
+      bool issued = false;
+      int64_t g = 0;  // accumulator tiles so far (ping-pong over two)
+      int seg = 0;
+      const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+      for (int64_t w = w_begin; w < w_end && ok; ++seg) {
+        const Seg sg = segment_at(w, w_end, n_tiles, qblocks, ca);
+        const int t0 = sg.t0, t1 = sg.t1;
+        w += t1 - t0;
+        if (!mbar_wait_warp(&bars->a_full, (uint32_t)(seg & 1), abort, err, 2)) {
+          ok = false;
+          break;
+        }
+        for (int t = t0; t < t1; ++t, ++g) {
+          const int b = (int)(g & 1);
+          const uint32_t use = (uint32_t)(g >> 1);
+          if (!mbar_wait_warp(&bars->tempty[b], (use & 1) ^ 1, abort, err, 3)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint64_t a0 = sw128_desc(sA0 + kb * kABytes);
-          const uint64_t b0 = sw128_desc(sB0 + stage * kBBytes);
-          const int kmax = kb == kb_count - 1 ? k_last : kMmaPerStage;
-          if (elect_one()) {
-            // the next 32 bytes of K: 2 more in the descriptors' 16-byte units
-#pragma unroll
-            for (int kk = 0; kk < kMmaPerStage; ++kk)
-              if (kk < kmax) {
-                if constexpr (kE4M3)
-                  umma_e4m3(d, a0 + kk * 2, b0 + kk * 2, (kb | kk) != 0 ? 1u : 0u);
-                else
-                  umma_bf16(d, a0 + kk * 2, b0 + kk * 2, (kb | kk) != 0 ? 1u : 0u);
-              }
-            umma_commit(&bars->empty[stage]);
-            if (kb == kb_count - 1) umma_commit(&bars->tfull[b]);
+          const uint32_t d = tmem + (uint32_t)(b * kTN);
+          for (int kb = 0; kb < kb_count; ++kb) {
+            if (!mbar_wait_warp(&bars->full[stage], phase, abort, err, 4)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t a0 = sw128_desc(sA0 + kb * kABytes);
+            const uint64_t b0 = sw128_desc(sB0 + stage * kBBytes);
+            const int kmax = kb == kb_count - 1 ? k_last : kMmaPerStage;
+            if (elect_one()) {
+              // the next 32 bytes of K: 2 more in the descriptors' 16-byte units
+  #pragma unroll
+              for (int kk = 0; kk < kMmaPerStage; ++kk)
+                if (kk < kmax) umma_bf16(d, a0 + kk * 2, b0 + kk * 2, (kb | kk) != 0 ? 1u : 0u);
+              umma_commit(&bars->empty[stage]);
+              if (kb == kb_count - 1) umma_commit(&bars->tfull[b]);
+            }
+            __syncwarp();
+            issued = true;
+            if (++stage == nstages) {
+              stage = 0;
+              phase ^= 1;
+            }
           }
-          __syncwarp();
-          issued = true;
-          if (++stage == nstages) {
-            stage = 0;
-            phase ^= 1;
-          }
+          if (!ok) break;
         }
-        if (!ok) break;
+        if (ok && elect_one()) umma_commit(&bars->a_empty);  // A may be replaced once these MMAs complete
+        __syncwarp();
       }
-      if (ok && elect_one()) umma_commit(&bars->a_empty);  // A may be replaced once these MMAs complete
-      __syncwarp();
-    }
-    if (!ok && issued) {  // wait for the MMAs issued before TMEM is freed (bounded)
-      if (elect_one()) umma_commit(&bars->drain);
-      __syncwarp();
-      mbar_wait(&bars->drain, 0, nullptr, nullptr, 0);
+      if (!ok && issued) {  // wait for the MMAs issued before TMEM is freed (bounded)
+        if (elect_one()) umma_commit(&bars->drain);
+        __syncwarp();
+        mbar_wait(&bars->drain, 0, nullptr, nullptr, 0);
+      }
     }
   } else {
-    const int ew = warp - 2;   // epilogue warp 0..7
+    if constexpr (!kCollect) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsHigh));
+    const int ew = warp - 4;   // epilogue warp 0..7
     const int q = warp & 3;    // TMEM lane quarter this warp may access
     const int h = ew >> 2;     // column slice of every tile
     const int r = q * 32 + lane;
@@ -554,7 +551,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
           }
           release();
         } else {
-          fold_slice<C, 4>(tb, (uint32_t)jb, (uint32_t)n, (uint32_t)i_self, L, release);
+          fold_slice<C>(tb, (uint32_t)jb, (uint32_t)n, (uint32_t)i_self, L, release);
         }
       }
       if (!kCollect && ok) {
@@ -615,15 +612,6 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 constexpr int kPairRows = 2 * kTM;             // query rows of a pair's block
 constexpr int kPairBBytes = kTN / 2 * kTKB;    // 16 KB of keys per stage and CTA
 constexpr int kPairMaxStages = 12;
-// Three warpgroups: the producer, the MMA issuer and two idle warps, then the
-// eight epilogue warps.  What decides whether the MMAs wait is how soon an
-// accumulator comes back, so the epilogue takes all 128 columns of its slice
-// into registers before it looks at them; the first warpgroup gives up its
-// registers for that (setmaxnreg: 128 x 64 + 256 x 216 = 63,488 of the
-// 384 x 168 = 64,512 the block is launched with).
-constexpr int kPairThreads = 128 + 32 * kEpiWarps;
-constexpr int kPairRegsLow = 64, kPairRegsHigh = 216;
-
 struct __align__(8) PairBars {
   uint64_t full[kPairMaxStages];   // leader: both CTAs' halves of the stage have landed
   uint64_t empty[kPairMaxStages];  // each CTA: the MMAs that read the stage have completed
@@ -697,7 +685,7 @@ __device__ __forceinline__ void pair_arrive(uint32_t bar) {
 // ...; past the last one the keys are padding), and row i leaves two lists per
 // share, at (i * shares + share) * kCandC; qblocks counts (block, share) pairs.
 template <bool kE4M3>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
 k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
            int64_t n_pad, int64_t qblocks, int kb_count, int k_last, int nstages, float* __restrict__ cand_val,
            int32_t* __restrict__ cand_idx, const float* __restrict__ out_scale, float* __restrict__ part_val,
@@ -750,7 +738,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
   const uint32_t tmem = bars->tmem_base;
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPairRegsLow));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
     if (warp == 0) {
       int stage = 0;
       uint32_t phase = 0;
@@ -890,7 +878,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPairRegsHigh));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsHigh));
     const int q = warp & 3;          // TMEM lane quarter this warp may access
     const int h = (warp - 4) >> 2;   // column half of every tile
     const int r = q * 32 + lane;
@@ -930,7 +918,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
           __syncwarp();
           if (lane == 0) pair_arrive(tempty0 + (uint32_t)(b * sizeof(uint64_t)));
         };
-        fold_slice<C, 8>(tb, jb, (uint32_t)n, (uint32_t)i, L, release);
+        fold_slice<C>(tb, jb, (uint32_t)n, (uint32_t)i, L, release);
       }
       if (!ok) break;
       L.flush((uint32_t)n, (uint32_t)i);
@@ -1469,14 +1457,14 @@ __global__ void k_gather_rows(const uint8_t* __restrict__ x, int row_bytes, cons
 
 // One persistent CTA per SM (at most one per work item); list mode adds the
 // partial-list area and the merge of split query blocks.
-template <bool kCollect, bool kE4M3>
+template <bool kCollect>
 ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& tb, int64_t n, int64_t n_pad,
                        int64_t n_rows, int kb_count, int d, float* cand_val, int32_t* cand_idx,
                        const float* out_scale, const CollectArgs& ca, int32_t* err, cudaStream_t s,
                        int key_stride = 1) {
-  // MMAs over the last 128-byte feature block: K = 16 features (BF16) or 32
-  // (E4M3) each; the padding past d is zero and needs none
-  const int per_kb = kE4M3 ? 128 : 64, per_mma = kE4M3 ? 32 : 16;
+  // MMAs over the last 128-byte feature block: K = 16 features each; the
+  // padding past d is zero and needs none
+  const int per_kb = 64, per_mma = 16;
   const int rem = d - per_kb * (kb_count - 1);
   const int k_last = (rem >= 1 && rem <= per_kb) ? (int)ceil_div(rem, per_mma) : kMmaPerStage;
   int nstages;
@@ -1500,8 +1488,8 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
   // on every call: a key order that moves with timing resolves exact score
   // ties differently)
   if (key_stride == 1 && !ca.blk_ptr && !ca.no_self) ANCKA_TRY(ws.zeros(&tick, 1));
-  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_tc<kCollect, kE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_knn_tc<kCollect, kE4M3><<<(unsigned)ctas, kThreads, smem, s>>>(ta, tb, n, n_pad, qblocks, kb_count, k_last,
+  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_tc<kCollect>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_knn_tc<kCollect><<<(unsigned)ctas, kTcThreads, smem, s>>>(ta, tb, n, n_pad, qblocks, kb_count, k_last,
                                                                    nstages, key_stride, cand_val, cand_idx,
                                                                    out_scale, part_val, part_idx, ca, tick, err);
   ANCKA_LAUNCHED();
@@ -1543,7 +1531,7 @@ ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap
   ANCKA_TRY(ws.alloc(&part_idx, (size_t)pairs * 2 * kPairRows * kCandC));
   ANCKA_TRY(ws.zeros(&tick, 1));
   ANCKA_CUDA(cudaFuncSetAttribute(k_knn_pair<kE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_knn_pair<kE4M3><<<(unsigned)(2 * pairs), kPairThreads, smem, s>>>(
+  k_knn_pair<kE4M3><<<(unsigned)(2 * pairs), kTcThreads, smem, s>>>(
       ta, tb, n, n_pad, qblocks, kb_count, k_last, nstages, cand_val, cand_idx, out_scale, part_val, part_idx,
       a_rows, n_rows, shares, tick, err);
   ANCKA_LAUNCHED();
@@ -1575,7 +1563,7 @@ ancka_status knn_candidates_bf16_sym(Workspace& ws, const PrepOut& pr, int64_t n
   ANCKA_TRY(ws.alloc(&sv, (size_t)n * kCandC));
   ANCKA_TRY(ws.alloc(&si, (size_t)n * kCandC));
   CollectArgs none{};
-  const ancka_status st = launch_tc<false, false>(ws, ta, tb, n, pr.n_pad, n, kb_count, pr.d, sv, si, nullptr, none,
+  const ancka_status st = launch_tc<false>(ws, ta, tb, n, pr.n_pad, n, kb_count, pr.d, sv, si, nullptr, none,
                                                   err, s, kSymStride);
   if (st != ANCKA_OK) return st;
   // 2. thresholds
@@ -1714,7 +1702,7 @@ ancka_status knn_lists_bf16(Workspace& ws, const __nv_bfloat16* a, int64_t a_row
   ca.blk_tiles = blk_tiles;
   ca.blk_work = blk_work;
   ca.no_self = no_self ? 1 : 0;
-  return launch_tc<false, false>(ws, ta, tb, n_keys, keys_pad, n_rows, kb_count, d, cand_val, cand_idx, nullptr, ca,
+  return launch_tc<false>(ws, ta, tb, n_keys, keys_pad, n_rows, kb_count, d, cand_val, cand_idx, nullptr, ca,
                                  err, s);
 }
 
@@ -1731,7 +1719,7 @@ ancka_status knn_collect_bf16(Workspace& ws, const PrepOut& pr, int64_t n, const
   ANCKA_TRY(make_map(&ta, af, pr.dp, n_a_pad, kTM, 2));
   ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN, 2));
   CollectArgs ca{rows, n_a, thr, cnt, buf, cap};
-  return launch_tc<true, false>(ws, ta, tb, n, pr.n_pad, n_a, kb_count, pr.d, nullptr, nullptr, nullptr, ca, err, s);
+  return launch_tc<true>(ws, ta, tb, n, pr.n_pad, n_a, kb_count, pr.d, nullptr, nullptr, nullptr, ca, err, s);
 }
 
 }  // namespace ancka
