@@ -16,6 +16,7 @@
 //              in BF16, split over the node range);
 //   update     Adam with FP32 master weights; W1^T refreshed in BF16.
 // Reductions over nodes use float-float partial sums in a fixed order.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -39,55 +40,87 @@ __global__ void k_unit_rows(const float* __restrict__ X, int64_t n, int d, int l
   for (int c = lane; c < ld; c += 32) U[i * ld + c] = c < d ? x[c] * inv : 0.f;
 }
 
-// A[i, :] = [U_i | PU_i | 0] in BF16 (n x kp); At = A^T (kp x n_pad, zero for
-// i >= n) when requested
-__global__ void k_pack_features(const float* __restrict__ U, const float* __restrict__ PU, int64_t n, int d, int ld,
-                                int kp, __nv_bfloat16* __restrict__ A) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * kp) return;
-  const int64_t i = t / kp;
-  const int c = (int)(t % kp);
-  const float v = c < d ? U[i * ld + c] : (c < 2 * d ? PU[i * ld + c - d] : 0.f);
-  A[t] = __float2bfloat16_rn(v);
-}
-
-// 32 x 32 tile transpose of a BF16 matrix (rows x cols) into (cols x rows_pad)
-__global__ void k_transpose_bf16(const __nv_bfloat16* __restrict__ A, int64_t rows, int cols, int64_t rows_pad,
-                                 __nv_bfloat16* __restrict__ At) {
-  __shared__ __nv_bfloat16 tile[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32;
-  const int c0 = blockIdx.y * 32;
-  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
-    const int64_t r = r0 + q;
-    const int c = c0 + threadIdx.x;
-    tile[q][threadIdx.x] = (r < rows && c < cols) ? A[r * cols + c] : __float2bfloat16_rn(0.f);
+// A[i, :] = [U_i | PU_i | 0] in BF16 (n_rows x kp, zero for i >= n) and, when
+// requested, At = A^T (kp x n_pad): 64 x 64 tiles through shared memory, so
+// that the features are read once and both copies are written in 128-byte
+// rows.  Bound by HBM (820 MB at n = 200,000, d = 256); a thread per element
+// with its own divisions, then a transpose, took 0.51 ms there.
+__global__ void __launch_bounds__(256)
+k_pack_features(const float* __restrict__ U, const float* __restrict__ PU, int64_t n, int d, int ld, int kp,
+                int64_t n_pad, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ At) {
+  __shared__ __nv_bfloat16 tile[64][66];
+  const int64_t r0 = (int64_t)blockIdx.x * 64;
+  const int c0 = blockIdx.y * 64, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ca = c0 + lane, cb = ca + 32;
+  float v[8][2];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int64_t i = r0 + w + 8 * q;
+    const float* u = U + i * ld;
+    const float* pu = PU + i * ld - d;
+    v[q][0] = i < n && ca < 2 * d ? (ca < d ? u[ca] : pu[ca]) : 0.f;
+    v[q][1] = i < n && cb < 2 * d ? (cb < d ? u[cb] : pu[cb]) : 0.f;
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    tile[w + 8 * q][lane] = __float2bfloat16_rn(v[q][0]);
+    tile[w + 8 * q][lane + 32] = __float2bfloat16_rn(v[q][1]);
   }
   __syncthreads();
-  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
-    const int c = c0 + q;
-    const int64_t r = r0 + threadIdx.x;
-    if (c < cols && r < rows_pad) At[(int64_t)c * rows_pad + r] = tile[threadIdx.x][q];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int r = w + 8 * q;
+    const __nv_bfloat162 p = __halves2bfloat162(tile[r][2 * lane], tile[r][2 * lane + 1]);
+    *reinterpret_cast<__nv_bfloat162*>(A + (r0 + r) * kp + c0 + 2 * lane) = p;
+  }
+  if (!At || r0 >= n_pad) return;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int c = w + 8 * q;
+    const __nv_bfloat162 p = __halves2bfloat162(tile[2 * lane][c], tile[2 * lane + 1][c]);
+    *reinterpret_cast<__nv_bfloat162*>(At + (int64_t)(c0 + c) * n_pad + r0 + 2 * lane) = p;
   }
 }
 
-// W = H W2 + b2, one warp per row (fixed-order butterfly per output)
-__global__ void k_mlp_out(const float* __restrict__ H, int64_t n, const float* __restrict__ W2,
-                          const float* __restrict__ b2, int k, float* __restrict__ W, int ldw) {
-  extern __shared__ float w2s[];  // kHidden x k
-  for (int e = threadIdx.x; e < kHidden * k; e += blockDim.x) w2s[e] = W2[e];
+// W = H W2 + b2, one warp per row, rows grid-stride.  A lane sums its 8 hidden
+// units into 32 outputs, then five levels each halve the outputs a lane keeps
+// (the additions of a butterfly per output, 31 shuffles instead of 160), which
+// leaves output c in lane c.  W2 is kept transposed in shared memory (its
+// rows, k floats apart, collided on the banks) and loaded once per CTA, not
+// once per 8 rows: 0.54 ms before at n = 200,000, k = 20.
+__global__ void __launch_bounds__(256)
+k_mlp_out(const float* __restrict__ H, int64_t n, const float* __restrict__ W2, const float* __restrict__ b2, int k,
+          float* __restrict__ W, int ldw) {
+  extern __shared__ float w2s[];  // k x kHidden
+  for (int e = threadIdx.x; e < kHidden * k; e += blockDim.x) w2s[(e % k) * kHidden + e / k] = W2[e];
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= n) return;
-  float h[kHidden / 32];
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += step) {
+    float h[kHidden / 32];
 #pragma unroll
-  for (int j = 0; j < kHidden / 32; ++j) h[j] = H[i * kHidden + lane + 32 * j];
-  for (int c = 0; c < k; ++c) {
-    float acc = 0.f;
+    for (int j = 0; j < kHidden / 32; ++j) h[j] = H[i * kHidden + lane + 32 * j];
+    for (int c0 = 0; c0 < k; c0 += 32) {
+      float v[32];
 #pragma unroll
-    for (int j = 0; j < kHidden / 32; ++j) acc = fmaf(h[j], w2s[(lane + 32 * j) * k + c], acc);
-    acc = warp_sum(acc);
-    if (lane == 0) W[i * ldw + c] = acc + b2[c];
+      for (int c = 0; c < 32; ++c) {
+        v[c] = 0.f;
+        if (c0 + c < k) {
+#pragma unroll
+          for (int j = 0; j < kHidden / 32; ++j) v[c] = fmaf(h[j], w2s[(c0 + c) * kHidden + lane + 32 * j], v[c]);
+        }
+      }
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int c = 0; c < off; ++c) {
+          const float send = up ? v[c] : v[c + off], keep = up ? v[c + off] : v[c];
+          v[c] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+      }
+      if (c0 + lane < k) W[i * ldw + c0 + lane] = v[0] + b2[c0 + lane];
+    }
   }
 }
 
@@ -101,51 +134,97 @@ __device__ __forceinline__ void ffa(float& hi, float& lo, float bh, float bl) {
 }
 
 // partial[blk][a][b] = sum over the CTA's rows of X[r, a] Y[r, b] (X null:
-// ones, p = 1), FP32 within 32-row tiles, float-float across tiles.  Thread a
-// owns row a of the result, columns in chunks of 16.
+// ones, p = 1), FP32 within 32-row tiles, float-float across tiles.  A thread
+// owns N blocks of one row a and four columns of the result (block e: a = e mod
+// p, columns 4 (e / p) ..), whose tile values are one load of X and one
+// 16-byte load of Y per row; a tile is staged once for all columns.  (A thread
+// per row a with 16 columns at a time left 236 of 256 threads idle for the
+// k x k products and staged H twice: 1.6 ms for the four products of a step at
+// n = 200,000, k = 20.)
 constexpr int kXtyRows = 32;
-__global__ void __launch_bounds__(256)
+template <int N>
+__global__ void __launch_bounds__(256, 2)
 k_xty_partial(const float* __restrict__ X, int ldx, const float* __restrict__ Y, int ldy, int64_t n, int p, int q,
               float2* __restrict__ partial) {
-  extern __shared__ float xs[];  // kXtyRows x (p + q)
-  float* ys = xs + kXtyRows * p;
+  extern __shared__ float4 xty_smem[];  // kXtyRows x q4 float4 of Y, then kXtyRows x p floats of X
+  const int q4 = (q + 3) / 4;
+  float4* ys4 = xty_smem;
+  float* ys = reinterpret_cast<float*>(xty_smem);
+  float* xs = ys + kXtyRows * 4 * q4;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per;
   const int64_t r1 = (r0 + per < n) ? r0 + per : n;
-  const int a = threadIdx.x;
-  for (int b0 = 0; b0 < q; b0 += 16) {
-    float hi[16], lo[16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int base = 0; base < p * q4; base += 256 * N) {
+    int ea[N], eg[N];
+    float hi[N][4], lo[N][4];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) hi[e] = lo[e] = 0.f;
+    for (int m = 0; m < N; ++m) {
+      const int e = base + threadIdx.x + 256 * m;
+      ea[m] = e % p;
+      eg[m] = e < p * q4 ? e / p : 0;  // past the last block: a valid one, not written
+#pragma unroll
+      for (int c = 0; c < 4; ++c) hi[m][c] = lo[m][c] = 0.f;
+    }
     for (int64_t rb = r0; rb < r1; rb += kXtyRows) {
       const int rows = (int)((r1 - rb) < kXtyRows ? (r1 - rb) : kXtyRows);
       __syncthreads();
-      for (int e = threadIdx.x; e < kXtyRows * p; e += blockDim.x) {
-        const int r = e / p, c = e % p;
-        xs[e] = r < rows ? (X ? X[(rb + r) * ldx + c] : 1.f) : 0.f;
-      }
-      for (int e = threadIdx.x; e < kXtyRows * q; e += blockDim.x) {
-        const int r = e / q, c = e % q;
-        ys[e] = r < rows ? Y[(rb + r) * ldy + c] : 0.f;
+      for (int r = warp; r < rows; r += 8) {
+        if (X) {
+#pragma unroll 8
+          for (int c = lane; c < p; c += 32) xs[r * p + c] = X[(rb + r) * ldx + c];
+        } else if (lane == 0) {
+          xs[r] = 1.f;
+        }
+        for (int c = lane; c < 4 * q4; c += 32) ys[r * 4 * q4 + c] = c < q ? Y[(rb + r) * ldy + c] : 0.f;
       }
       __syncthreads();
-      if (a < p) {
-        float acc[16];
+      float acc[N][4];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-        for (int r = 0; r < rows; ++r) {
-          const float xa = xs[r * p + a];
+      for (int m = 0; m < N; ++m)
 #pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (b0 + e < q) acc[e] = fmaf(xa, ys[r * q + b0 + e], acc[e]);
+        for (int c = 0; c < 4; ++c) acc[m][c] = 0.f;
+#pragma unroll 2
+      for (int r = 0; r < rows; ++r) {
+#pragma unroll
+        for (int m = 0; m < N; ++m) {
+          const float xa = xs[r * p + ea[m]];
+          const float4 y = ys4[r * q4 + eg[m]];
+          acc[m][0] = fmaf(xa, y.x, acc[m][0]);
+          acc[m][1] = fmaf(xa, y.y, acc[m][1]);
+          acc[m][2] = fmaf(xa, y.z, acc[m][2]);
+          acc[m][3] = fmaf(xa, y.w, acc[m][3]);
         }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) ffa(hi[e], lo[e], acc[e], 0.f);
       }
+#pragma unroll
+      for (int m = 0; m < N; ++m)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ffa(hi[m][c], lo[m][c], acc[m][c], 0.f);
     }
-    if (a < p)
-      for (int e = 0; e < 16 && b0 + e < q; ++e)
-        partial[((int64_t)blockIdx.x * p + a) * q + b0 + e] = make_float2(hi[e], lo[e]);
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+      if (base + threadIdx.x + 256 * m >= p * q4) continue;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (4 * eg[m] + c < q)
+          partial[((int64_t)blockIdx.x * p + ea[m]) * q + 4 * eg[m] + c] = make_float2(hi[m][c], lo[m][c]);
+    }
+  }
+}
+
+// sum over blocks (in order) of entry t of m entries per block; sixteen loads
+// in flight (one at a time, the 304 blocks took 44 us)
+__device__ __forceinline__ void sum_partials(const float2* __restrict__ part, int nblk, int64_t m, int t, float& hi,
+                                             float& lo) {
+  hi = 0.f;
+  lo = 0.f;
+  for (int b0 = 0; b0 < nblk; b0 += 16) {
+    float2 v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = b0 + u < nblk ? part[(int64_t)(b0 + u) * m + t] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (b0 + u < nblk) ffa(hi, lo, v[u].x, v[u].y);
   }
 }
 
@@ -153,11 +232,8 @@ k_xty_partial(const float* __restrict__ X, int ldx, const float* __restrict__ Y,
 __global__ void k_xty_reduce(const float2* __restrict__ partial, int nblk, int p, int q, double* __restrict__ out) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p * q) return;
-  float hi = 0.f, lo = 0.f;
-  for (int b = 0; b < nblk; ++b) {
-    const float2 v = partial[(int64_t)b * p * q + t];
-    ffa(hi, lo, v.x, v.y);
-  }
+  float hi, lo;
+  sum_partials(partial, nblk, (int64_t)p * q, t, hi, lo);
   out[t] = (double)hi + (double)lo;
 }
 
@@ -168,9 +244,14 @@ ancka_status xty(Workspace& ws, const float* X, int ldx, const float* Y, int ldy
   const int nb = xty_blocks(n);
   float2* part;
   ANCKA_TRY(ws.alloc(&part, (size_t)nb * p * q));
-  const size_t smem = (size_t)kXtyRows * (p + q) * sizeof(float);
-  ANCKA_CUDA(cudaFuncSetAttribute(k_xty_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_xty_partial<<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
+  const int blocks = p * ((q + 3) / 4);  // p <= kHidden and q <= 64: shared memory <= 41 KB
+  const size_t smem = (size_t)kXtyRows * (p + 4 * ((q + 3) / 4)) * sizeof(float);
+  if (blocks <= 256)
+    k_xty_partial<1><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
+  else if (blocks <= 1024)
+    k_xty_partial<4><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
+  else  // six blocks fill the registers two CTAs an SM leave a thread
+    k_xty_partial<6><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
   ANCKA_LAUNCHED();
   k_xty_reduce<<<(unsigned)ceil_div(p * q, 128), 128, 0, s>>>(part, nb, p, q, out);
   ANCKA_LAUNCHED();
@@ -178,51 +259,60 @@ ancka_status xty(Workspace& ws, const float* X, int ldx, const float* Y, int ldy
 }
 
 // One CTA, FP64: from G = W^T W and M = Q_t^T W (k x k), the loss and the
-// coefficient matrices of dL/dW = W C1 + Q_t C2.  G^-1 by Cholesky; a
-// non-positive pivot sets *status.
-__global__ void k_warm_coeffs(const double* __restrict__ G, const double* __restrict__ M, int k, double n, double lam,
-                              float* __restrict__ C1, float* __restrict__ C2, double* __restrict__ loss,
-                              int32_t* __restrict__ status) {
+// coefficient matrices of dL/dW = W C1 + Q_t C2.  G = L L^T by a right-looking
+// Cholesky and, in the same steps, Y = L^-1 by Gauss-Jordan elimination on
+// [L | I], so that a step is one reciprocal root and a few dependent FP64
+// operations across the CTA (with serial pivots, divisions and a thread per
+// column of the back substitution the kernel took 240 us at k = 20); G^-1 =
+// Y^T Y.  A non-positive pivot sets *status.
+constexpr int kCoeffThreads = 512;
+__global__ void __launch_bounds__(kCoeffThreads)
+k_warm_coeffs(const double* __restrict__ G, const double* __restrict__ M, int k, double n, double lam,
+              float* __restrict__ C1, float* __restrict__ C2, double* __restrict__ loss,
+              int32_t* __restrict__ status) {
   extern __shared__ double sm[];
-  double* R = sm;               // k x k Cholesky factor (upper)
+  double* R = sm;               // k x k: G's trailing block, then the columns of L (row j: column j of L)
   double* Gi = R + k * k;       // G^-1
   double* T1 = Gi + k * k;      // M^T M
-  double* T2 = T1 + k * k;      // G^-1 M^T M
+  double* T2 = T1 + k * k;      // Y = L^-1, then G^-1 M^T M
   double* Sm = T2 + k * k;      // S
+  __shared__ double rinv;
   const int kk = k * k;
-  for (int e = threadIdx.x; e < kk; e += blockDim.x) R[e] = 0.0;
+  for (int e = threadIdx.x; e < kk; e += blockDim.x) {
+    R[e] = G[e];
+    T2[e] = e / k == e % k ? 1.0 : 0.0;
+  }
   __syncthreads();
-  for (int j = 0; j < k; ++j) {  // G = R^T R
+  for (int j = 0; j < k; ++j) {
     if (threadIdx.x == 0) {
-      double dgn = G[j * k + j];
-      for (int m = 0; m < j; ++m) dgn -= R[m * k + j] * R[m * k + j];
-      if (!(dgn > 0.0)) {
+      double d = R[j * k + j];
+      if (!(d > 0.0)) {
         *status = 1;
-        dgn = 1e-300;
+        d = 1e-300;
       }
-      R[j * k + j] = sqrt(dgn);
+      rinv = 1.0 / sqrt(d);
     }
     __syncthreads();
-    for (int c = j + 1 + threadIdx.x; c < k; c += blockDim.x) {
-      double v = G[j * k + c];
-      for (int m = 0; m < j; ++m) v -= R[m * k + j] * R[m * k + c];
-      R[j * k + c] = v / R[j * k + j];
+    const double ri = rinv;
+    // row j of L^T (columns > j) and of Y (columns <= j) times 1 / L_jj
+    for (int c = threadIdx.x; c < k; c += blockDim.x) {
+      if (c > j) R[j * k + c] *= ri;
+      else T2[j * k + c] *= ri;
+    }
+    __syncthreads();
+    const int m = k - j - 1;  // later rows
+    for (int e = threadIdx.x; e < m * k; e += blockDim.x) {
+      const int i = j + 1 + e / k, c = e % k;
+      const double lij = R[j * k + i];
+      if (c <= j) T2[i * k + c] = fma(-lij, T2[j * k + c], T2[i * k + c]);
+      else if (c >= i) R[i * k + c] = fma(-lij, R[j * k + c], R[i * k + c]);
     }
     __syncthreads();
   }
-  // G^-1 = R^-1 R^-T: column c of R^-1 by back substitution (thread c), then Gi
-  for (int c = threadIdx.x; c < k; c += blockDim.x) {
-    for (int i = k - 1; i >= 0; --i) {  // X = R^-1 stored in T2 (column c)
-      double v = (i == c) ? 1.0 : 0.0;
-      for (int m = i + 1; m < k; ++m) v -= R[i * k + m] * T2[m * k + c];
-      T2[i * k + c] = v / R[i * k + i];
-    }
-  }
-  __syncthreads();
   for (int e = threadIdx.x; e < kk; e += blockDim.x) {
     const int a = e / k, b = e % k;
     double v = 0.0;
-    for (int m = 0; m < k; ++m) v += T2[a * k + m] * T2[b * k + m];
+    for (int m = max(a, b); m < k; ++m) v += T2[m * k + a] * T2[m * k + b];
     Gi[e] = v;
     double w = 0.0;
     for (int m = 0; m < k; ++m) w += M[m * k + a] * M[m * k + b];
@@ -285,44 +375,58 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
 // dZ1 = (dW W2^T) * GELU'(Z1) in tiles of 32 rows (a CTA takes tiles
 // blockIdx.x, blockIdx.x + gridDim.x, ...), thread j = hidden unit; written
 // transposed in BF16 (dZ1t: kHidden x n_pad) and summed per CTA for db1
-// (float-float partials)
+// (float-float partials).  KQ: 16-byte groups of a row of dW (4 KQ >= k, zero
+// padded), so that a row costs KQ loads of dW and 4 KQ FMAs instead of 64
+// predicated ones of each; eight rows' Z1 are loaded ahead.
 constexpr int kDzRows = 32;
-__global__ void __launch_bounds__(kHidden)
+template <int KQ>
+__global__ void __launch_bounds__(kHidden, 2)
 k_dz1(const float* __restrict__ dW, int ldw, const float* __restrict__ Z1, const float* __restrict__ W2, int k,
       int64_t n, int64_t n_pad, __nv_bfloat16* __restrict__ dZ1t, float2* __restrict__ db1_part) {
-  __shared__ float dws[kDzRows][64];
-  __shared__ __nv_bfloat16 tile[kHidden][kDzRows + 2];
+  __shared__ float4 dws[kDzRows][KQ];
+  __shared__ __nv_bfloat162 tile[kHidden][kDzRows / 2 + 1];
   const int j = threadIdx.x;
-  float w2[64];
+  float w2[4 * KQ];
 #pragma unroll
-  for (int c = 0; c < 64; ++c) w2[c] = c < k ? W2[j * k + c] : 0.f;
+  for (int c = 0; c < 4 * KQ; ++c) w2[c] = c < k ? W2[j * k + c] : 0.f;
   float hi = 0.f, lo = 0.f;
   const int64_t ntiles = ceil_div(n_pad, (int64_t)kDzRows);
   for (int64_t tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
     const int64_t r0 = tl * kDzRows;
     __syncthreads();
-    for (int e = threadIdx.x; e < kDzRows * k; e += blockDim.x) {
-      const int r = e / k, c = e % k;
-      dws[r][c] = (r0 + r < n) ? dW[(r0 + r) * ldw + c] : 0.f;
+    for (int e = threadIdx.x; e < kDzRows * 4 * KQ; e += blockDim.x) {
+      const int r = e / (4 * KQ), c = e % (4 * KQ);
+      reinterpret_cast<float*>(dws)[e] = (c < k && r0 + r < n) ? dW[(r0 + r) * ldw + c] : 0.f;
     }
     __syncthreads();
-    for (int r = 0; r < kDzRows; ++r) {
-      float dz = 0.f;
-      if (r0 + r < n) {
+#pragma unroll 1
+    for (int rb = 0; rb < kDzRows; rb += 8) {
+      float z[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) z[u] = r0 + rb + u < n ? Z1[(r0 + rb + u) * kHidden + j] : 0.f;
+      float dz[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
         float dh = 0.f;
 #pragma unroll
-        for (int c = 0; c < 64; ++c)
-          if (c < k) dh = fmaf(dws[r][c], w2[c], dh);
-        dz = dh * gelu_grad_f(Z1[(r0 + r) * kHidden + j]);
+        for (int g = 0; g < KQ; ++g) {
+          const float4 v = dws[rb + u][g];
+          dh = fmaf(v.x, w2[4 * g], dh);
+          dh = fmaf(v.y, w2[4 * g + 1], dh);
+          dh = fmaf(v.z, w2[4 * g + 2], dh);
+          dh = fmaf(v.w, w2[4 * g + 3], dh);
+        }
+        dz[u] = r0 + rb + u < n ? dh * gelu_grad_f(z[u]) : 0.f;
+        ffa(hi, lo, dz[u], 0.f);
       }
-      ffa(hi, lo, dz, 0.f);
-      tile[j][r] = __float2bfloat16_rn(dz);
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) tile[j][(rb + u) / 2] = __floats2bfloat162_rn(dz[u], dz[u + 1]);
     }
     __syncthreads();
-    // row jj of dZ1t: 32 consecutive nodes
-    for (int e = threadIdx.x; e < kHidden * kDzRows; e += blockDim.x) {
-      const int jj = e / kDzRows, r = e % kDzRows;
-      if (r0 + r < n_pad) dZ1t[(int64_t)jj * n_pad + r0 + r] = tile[jj][r];
+    // row jj of dZ1t: 32 consecutive nodes (n_pad is a multiple of 64)
+    for (int e = threadIdx.x; e < kHidden * kDzRows / 2; e += blockDim.x) {
+      const int jj = e / (kDzRows / 2), r = e % (kDzRows / 2);
+      *reinterpret_cast<__nv_bfloat162*>(dZ1t + (int64_t)jj * n_pad + r0 + 2 * r) = tile[jj][r];
     }
   }
   db1_part[(int64_t)blockIdx.x * kHidden + j] = make_float2(hi, lo);
@@ -331,11 +435,8 @@ k_dz1(const float* __restrict__ dW, int ldw, const float* __restrict__ Z1, const
 __global__ void k_reduce_f2(const float2* __restrict__ part, int nblk, int m, float* __restrict__ out) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= m) return;
-  float hi = 0.f, lo = 0.f;
-  for (int b = 0; b < nblk; ++b) {
-    const float2 v = part[(int64_t)b * m + t];
-    ffa(hi, lo, v.x, v.y);
-  }
+  float hi, lo;
+  sum_partials(part, nblk, m, t, hi, lo);
   out[t] = hi + lo;
 }
 
@@ -379,22 +480,18 @@ ancka_status warm_features(Workspace& ws, const Walk& w, const float* X, int d, 
   const int64_t n = w.n;
   const int ld = (int)round_up(d, 4);
   const int kp = warm_kp(d);
-  ANCKA_CUDA(cudaMemsetAsync(A, 0, sizeof(__nv_bfloat16) * round_up(n, 128) * kp, s));
-  if (At) ANCKA_CUDA(cudaMemsetAsync(At, 0, sizeof(__nv_bfloat16) * round_up(kp, 128) * round_up(n, 64), s));
+  const int64_t n_pad = round_up(n, 64);
+  if (At && kp % 128 != 0)  // the rows past kp; the kernel writes the rest
+    ANCKA_CUDA(cudaMemsetAsync(At + (int64_t)kp * n_pad, 0, sizeof(__nv_bfloat16) * (round_up(kp, 128) - kp) * n_pad, s));
   float *U, *PU;
   ANCKA_TRY(ws.alloc(&U, (size_t)n * ld));
   ANCKA_TRY(ws.alloc(&PU, (size_t)n * ld));
   k_unit_rows<<<(unsigned)ceil_div(n * 32, 256), 256, 0, s>>>(X, n, d, ld, U);
   ANCKA_LAUNCHED();
   ANCKA_TRY(apply_topology(ws, w, U, ld, PU, s));
-  k_pack_features<<<(unsigned)ceil_div(n * kp, 256), 256, 0, s>>>(U, PU, n, d, ld, kp, A);
+  const dim3 grid((unsigned)(round_up(n, 128) / 64), (unsigned)(kp / 64));
+  k_pack_features<<<grid, 256, 0, s>>>(U, PU, n, d, ld, kp, n_pad, A, At);
   ANCKA_LAUNCHED();
-  if (At) {
-    const int64_t n_pad = round_up(n, 64);
-    dim3 grid((unsigned)ceil_div(n_pad, 32), (unsigned)ceil_div(kp, 32));
-    k_transpose_bf16<<<grid, dim3(32, 8), 0, s>>>(A, n, kp, n_pad, At);
-    ANCKA_LAUNCHED();
-  }
   return ANCKA_OK;
 }
 
@@ -408,7 +505,8 @@ ancka_status warm_forward(Workspace& ws, const __nv_bfloat16* A, int64_t n, int 
   ANCKA_TRY(gemm_bias_gelu(A, n, kp, W1t, b1, Z1, H, kHidden, err, s));
   const size_t smem = (size_t)kHidden * k * sizeof(float);
   ANCKA_CUDA(cudaFuncSetAttribute(k_mlp_out, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_mlp_out<<<(unsigned)ceil_div(n * 32, 256), 256, smem, s>>>(H, n, W2, b2, k, W, ldw);
+  // at most three CTAs an SM at k = 64 (64 KB each), so four waves at most
+  k_mlp_out<<<(unsigned)std::min<int64_t>(ceil_div(n, 8), 152 * 6), 256, smem, s>>>(H, n, W2, b2, k, W, ldw);
   ANCKA_LAUNCHED();
   return ANCKA_OK;
 }
@@ -452,7 +550,7 @@ ancka_status warm_train_step(Workspace& ws, const WarmStepArgs& a, cudaStream_t 
   ANCKA_TRY(xty(ws, a.Qt, a.ldq, W, ldw, n, k, k, M, s));
   const size_t csm = (size_t)5 * k * k * sizeof(double);
   ANCKA_CUDA(cudaFuncSetAttribute(k_warm_coeffs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-  k_warm_coeffs<<<1, 128, csm, s>>>(G, M, k, (double)n, (double)a.lam, C1, C2, a.loss_dev, a.status);
+  k_warm_coeffs<<<1, kCoeffThreads, csm, s>>>(G, M, k, (double)n, (double)a.lam, C1, C2, a.loss_dev, a.status);
   ANCKA_LAUNCHED();
   k_grad_w<<<(unsigned)ceil_div(n * k, 256), 256, (size_t)2 * k * k * sizeof(float), s>>>(W, ldw, a.Qt, a.ldq, n, k,
                                                                                            C1, C2, dW);
@@ -467,7 +565,8 @@ ancka_status warm_train_step(Workspace& ws, const WarmStepArgs& a, cudaStream_t 
   const int nb = (int)std::min<int64_t>(304, ceil_div(n_pad, (int64_t)kDzRows));
   float2* db1p;
   ANCKA_TRY(ws.alloc(&db1p, (size_t)nb * kHidden));
-  k_dz1<<<nb, kHidden, 0, s>>>(dW, ldw, Z1, a.W2, k, n, n_pad, dZ1t, db1p);
+  auto dz1 = k <= 8 ? k_dz1<2> : k <= 20 ? k_dz1<5> : k <= 32 ? k_dz1<8> : k <= 48 ? k_dz1<12> : k_dz1<16>;
+  dz1<<<nb, kHidden, 0, s>>>(dW, ldw, Z1, a.W2, k, n, n_pad, dZ1t, db1p);
   ANCKA_LAUNCHED();
   k_reduce_f2<<<1, kHidden, 0, s>>>(db1p, nb, kHidden, db1);
   ANCKA_LAUNCHED();
