@@ -145,12 +145,13 @@ constexpr int kXtyRows = 32;
 template <int N>
 __global__ void __launch_bounds__(256, 2)
 k_xty_partial(const float* __restrict__ X, int ldx, const float* __restrict__ Y, int ldy, int64_t n, int p, int q,
-              float2* __restrict__ partial) {
-  extern __shared__ float4 xty_smem[];  // kXtyRows x q4 float4 of Y, then kXtyRows x p floats of X
+              int stage_rows, float2* __restrict__ partial) {
+  // stage_rows (a multiple of kXtyRows) x q4 float4 of Y, then as many rows of p floats of X
+  extern __shared__ float4 xty_smem[];
   const int q4 = (q + 3) / 4;
   float4* ys4 = xty_smem;
   float* ys = reinterpret_cast<float*>(xty_smem);
-  float* xs = ys + kXtyRows * 4 * q4;
+  float* xs = ys + stage_rows * 4 * q4;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per;
   const int64_t r1 = (r0 + per < n) ? r0 + per : n;
@@ -166,9 +167,10 @@ k_xty_partial(const float* __restrict__ X, int ldx, const float* __restrict__ Y,
 #pragma unroll
       for (int c = 0; c < 4; ++c) hi[m][c] = lo[m][c] = 0.f;
     }
-    for (int64_t rb = r0; rb < r1; rb += kXtyRows) {
-      const int rows = (int)((r1 - rb) < kXtyRows ? (r1 - rb) : kXtyRows);
+    for (int64_t rb = r0; rb < r1; rb += stage_rows) {
+      const int rows = (int)((r1 - rb) < stage_rows ? (r1 - rb) : stage_rows);
       __syncthreads();
+#pragma unroll 4
       for (int r = warp; r < rows; r += 8) {
         if (X) {
 #pragma unroll 8
@@ -179,27 +181,30 @@ k_xty_partial(const float* __restrict__ X, int ldx, const float* __restrict__ Y,
         for (int c = lane; c < 4 * q4; c += 32) ys[r * 4 * q4 + c] = c < q ? Y[(rb + r) * ldy + c] : 0.f;
       }
       __syncthreads();
-      float acc[N][4];
+      for (int t0 = 0; t0 < rows; t0 += kXtyRows) {
+        const int t1 = min(rows, t0 + kXtyRows);
+        float acc[N][4];
 #pragma unroll
-      for (int m = 0; m < N; ++m)
+        for (int m = 0; m < N; ++m)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[m][c] = 0.f;
+          for (int c = 0; c < 4; ++c) acc[m][c] = 0.f;
 #pragma unroll 2
-      for (int r = 0; r < rows; ++r) {
+        for (int r = t0; r < t1; ++r) {
 #pragma unroll
-        for (int m = 0; m < N; ++m) {
-          const float xa = xs[r * p + ea[m]];
-          const float4 y = ys4[r * q4 + eg[m]];
-          acc[m][0] = fmaf(xa, y.x, acc[m][0]);
-          acc[m][1] = fmaf(xa, y.y, acc[m][1]);
-          acc[m][2] = fmaf(xa, y.z, acc[m][2]);
-          acc[m][3] = fmaf(xa, y.w, acc[m][3]);
+          for (int m = 0; m < N; ++m) {
+            const float xa = xs[r * p + ea[m]];
+            const float4 y = ys4[r * q4 + eg[m]];
+            acc[m][0] = fmaf(xa, y.x, acc[m][0]);
+            acc[m][1] = fmaf(xa, y.y, acc[m][1]);
+            acc[m][2] = fmaf(xa, y.z, acc[m][2]);
+            acc[m][3] = fmaf(xa, y.w, acc[m][3]);
+          }
         }
+#pragma unroll
+        for (int m = 0; m < N; ++m)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) ffa(hi[m][c], lo[m][c], acc[m][c], 0.f);
       }
-#pragma unroll
-      for (int m = 0; m < N; ++m)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ffa(hi[m][c], lo[m][c], acc[m][c], 0.f);
     }
 #pragma unroll
     for (int m = 0; m < N; ++m) {
@@ -212,29 +217,41 @@ k_xty_partial(const float* __restrict__ X, int ldx, const float* __restrict__ Y,
   }
 }
 
-// sum over blocks (in order) of entry t of m entries per block; sixteen loads
-// in flight (one at a time, the 304 blocks took 44 us)
-__device__ __forceinline__ void sum_partials(const float2* __restrict__ part, int nblk, int64_t m, int t, float& hi,
+// sum over blocks of entry t of m entries per block by eight neighbouring
+// lanes: lane u adds blocks u, u + 8, ... in order, then the lanes' sums are
+// combined in a fixed order (one thread per entry, one load in flight, took
+// 44 us for 304 blocks)
+constexpr int kSumLanes = 8;
+__device__ __forceinline__ void sum_partials(const float2* __restrict__ part, int nblk, int64_t m, int64_t t, float& hi,
                                              float& lo) {
   hi = 0.f;
   lo = 0.f;
-  for (int b0 = 0; b0 < nblk; b0 += 16) {
-    float2 v[16];
+  const int u = threadIdx.x % kSumLanes;
+#pragma unroll 8
+  for (int b = u; b < nblk; b += kSumLanes) {
+    const float2 v = t < m ? part[(int64_t)b * m + t] : make_float2(0.f, 0.f);
+    ffa(hi, lo, v.x, v.y);
+  }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) v[u] = b0 + u < nblk ? part[(int64_t)(b0 + u) * m + t] : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (b0 + u < nblk) ffa(hi, lo, v[u].x, v[u].y);
+  for (int off = 1; off < kSumLanes; off <<= 1) {
+    const float h2 = __shfl_xor_sync(0xffffffffu, hi, off), l2 = __shfl_xor_sync(0xffffffffu, lo, off);
+    if (u & off) {  // the lower lane's sum first in both
+      float h = h2, l = l2;
+      ffa(h, l, hi, lo);
+      hi = h;
+      lo = l;
+    } else {
+      ffa(hi, lo, h2, l2);
+    }
   }
 }
 
 // out[a][b] = sum over blocks (in order) of the partials, as double
 __global__ void k_xty_reduce(const float2* __restrict__ partial, int nblk, int p, int q, double* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p * q) return;
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) / kSumLanes;
   float hi, lo;
   sum_partials(partial, nblk, (int64_t)p * q, t, hi, lo);
-  out[t] = (double)hi + (double)lo;
+  if (t < p * q && threadIdx.x % kSumLanes == 0) out[t] = (double)hi + (double)lo;
 }
 
 int xty_blocks(int64_t n) { return (int)std::min<int64_t>(304, std::max<int64_t>(1, ceil_div(n, 256))); }
@@ -244,16 +261,23 @@ ancka_status xty(Workspace& ws, const float* X, int ldx, const float* Y, int ldy
   const int nb = xty_blocks(n);
   float2* part;
   ANCKA_TRY(ws.alloc(&part, (size_t)nb * p * q));
-  const int blocks = p * ((q + 3) / 4);  // p <= kHidden and q <= 64: shared memory <= 41 KB
-  const size_t smem = (size_t)kXtyRows * (p + 4 * ((q + 3) / 4)) * sizeof(float);
+  const int blocks = p * ((q + 3) / 4);
+  // as many 32-row tiles staged at a time as 47 KB hold, eight at most (one at
+  // p = 256, eight for the k x k products at k = 20, which waited for memory
+  // at every tile: 88 us each with one); p <= kHidden and q <= 64: 41 KB a tile
+  // at most
+  const size_t tile = (size_t)kXtyRows * (p + 4 * ((q + 3) / 4)) * sizeof(float);
+  const int tiles = (int)std::max<size_t>(1, std::min<size_t>(8, 47 * 1024 / tile));
+  const int sr = tiles * kXtyRows;
+  const size_t smem = tiles * tile;
   if (blocks <= 256)
-    k_xty_partial<1><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
+    k_xty_partial<1><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, sr, part);
   else if (blocks <= 1024)
-    k_xty_partial<4><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
+    k_xty_partial<4><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, sr, part);
   else  // six blocks fill the registers two CTAs an SM leave a thread
-    k_xty_partial<6><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, part);
+    k_xty_partial<6><<<nb, 256, smem, s>>>(X, ldx, Y, ldy, n, p, q, sr, part);
   ANCKA_LAUNCHED();
-  k_xty_reduce<<<(unsigned)ceil_div(p * q, 128), 128, 0, s>>>(part, nb, p, q, out);
+  k_xty_reduce<<<(unsigned)ceil_div((int64_t)p * q * kSumLanes, 128), 128, 0, s>>>(part, nb, p, q, out);
   ANCKA_LAUNCHED();
   return ANCKA_OK;
 }
@@ -335,18 +359,18 @@ k_warm_coeffs(const double* __restrict__ G, const double* __restrict__ M, int k,
     }
     Sm[e] = v;
     const double pen = G[e] / n - (a == b ? 1.0 : 0.0);
+    T1[e] = pen * pen;
     C1[e] = (float)(2.0 * v + 4.0 * lam / n * pen);
     C2[e] = (float)(-2.0 * u);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {  // a lane's entries in order, then a butterfly
     double tr = 0.0, pen = 0.0;
-    for (int a = 0; a < k; ++a) tr += T2[a * k + a];
-    for (int e = 0; e < kk; ++e) {
-      const double v = G[e] / n - ((e / k) == (e % k) ? 1.0 : 0.0);
-      pen += v * v;
-    }
-    *loss = (double)k - tr + lam * pen;
+    for (int a = threadIdx.x; a < k; a += 32) tr += T2[a * k + a];
+    for (int e = threadIdx.x; e < kk; e += 32) pen += T1[e];
+    tr = warp_sum_d(tr);
+    pen = warp_sum_d(pen);
+    if (threadIdx.x == 0) *loss = (double)k - tr + lam * pen;
   }
 }
 
@@ -433,11 +457,10 @@ k_dz1(const float* __restrict__ dW, int ldw, const float* __restrict__ Z1, const
 }
 
 __global__ void k_reduce_f2(const float2* __restrict__ part, int nblk, int m, float* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m) return;
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) / kSumLanes;
   float hi, lo;
   sum_partials(part, nblk, m, t, hi, lo);
-  out[t] = hi + lo;
+  if (t < m && threadIdx.x % kSumLanes == 0) out[t] = hi + lo;
 }
 
 __global__ void k_d2f(const double* __restrict__ a, int64_t m, float* __restrict__ b) {
@@ -568,7 +591,7 @@ ancka_status warm_train_step(Workspace& ws, const WarmStepArgs& a, cudaStream_t 
   auto dz1 = k <= 8 ? k_dz1<2> : k <= 20 ? k_dz1<5> : k <= 32 ? k_dz1<8> : k <= 48 ? k_dz1<12> : k_dz1<16>;
   dz1<<<nb, kHidden, 0, s>>>(dW, ldw, Z1, a.W2, k, n, n_pad, dZ1t, db1p);
   ANCKA_LAUNCHED();
-  k_reduce_f2<<<1, kHidden, 0, s>>>(db1p, nb, kHidden, db1);
+  k_reduce_f2<<<(unsigned)(kHidden * kSumLanes / 128), 128, 0, s>>>(db1p, nb, kHidden, db1);
   ANCKA_LAUNCHED();
   ANCKA_TRY(gemm_at_b(ws, a.At, a.kp, n_pad, dZ1t, dW1, a.err, s));
   if (a.grads) {  // gradients out (tests)
