@@ -812,6 +812,7 @@ ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int
     }
     int32_t* ex_rows = cl_rows;
     int32_t* ex_count = cl_count;
+    bool rows_left = true;  // as far as the host knows
     if (collect_prec == ANCKA_PREC_BF16) {
       // flagged rows: collect every key above the row's certified threshold
       // with the tensor-core contraction, then re-rank those exactly
@@ -824,9 +825,10 @@ ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int
         return ANCKA_ERR_TIMEOUT;
       }
       list_err = nullptr;  // checked
-      ANCKA_TRY(ws.zeros(&ex_count, 1));
-      ANCKA_TRY(ws.alloc(&ex_rows, (size_t)(nf > 0 ? nf : 1)));
+      rows_left = nf > 0;
       if (nf > 0) {
+        ANCKA_TRY(ws.zeros(&ex_count, 1));
+        ANCKA_TRY(ws.alloc(&ex_rows, (size_t)nf));
         constexpr int kCap = 2048;
         int32_t *cnt, *buf, *terr;
         ANCKA_TRY(ws.zeros(&cnt, (size_t)nf));
@@ -840,18 +842,20 @@ ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int
       }
     }
     // rows left: sliced over the whole GPU when few, one CTA per row when many
-    double* pv;
-    int32_t* pi;
-    ANCKA_TRY(ws.alloc(&pv, (size_t)kSlicedMaxRows * kSlices * K));
-    ANCKA_TRY(ws.alloc(&pi, (size_t)kSlicedMaxRows * kSlices * K));
-    k_exh_sliced<<<1216, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ex_rows, ex_count, pv, pi);
-    ANCKA_LAUNCHED();
-    k_exh_merge<<<8, 128, 0, s>>>(ex_rows, ex_count, K, pv, pi, out_idx, out_sim);
-    ANCKA_LAUNCHED();
-    k_knn_exhaustive<<<304, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ex_rows, ex_count, 0, out_idx,
-                                                   out_sim);
-    ANCKA_LAUNCHED();
-    ex_count_dev = ex_count;
+    if (rows_left) {
+      double* pv;
+      int32_t* pi;
+      ANCKA_TRY(ws.alloc(&pv, (size_t)kSlicedMaxRows * kSlices * K));
+      ANCKA_TRY(ws.alloc(&pi, (size_t)kSlicedMaxRows * kSlices * K));
+      k_exh_sliced<<<1216, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ex_rows, ex_count, pv, pi);
+      ANCKA_LAUNCHED();
+      k_exh_merge<<<8, 128, 0, s>>>(ex_rows, ex_count, K, pv, pi, out_idx, out_sim);
+      ANCKA_LAUNCHED();
+      k_knn_exhaustive<<<304, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ex_rows, ex_count, 0, out_idx,
+                                                     out_sim);
+      ANCKA_LAUNCHED();
+      ex_count_dev = ex_count;
+    }
   } else {
     const unsigned g = (unsigned)(n < 4096 ? n : 4096);
     k_knn_exhaustive<<<g, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, nullptr, nullptr, n, out_idx,
