@@ -233,10 +233,13 @@ __device__ __forceinline__ void fold_slice(uint32_t tb, uint32_t jb, uint32_t n,
   }
   release();
   const float thr = L.lv[C - 1];
+  float top = mx[0];
+#pragma unroll
+  for (int c = 1; c < kChunks; ++c) top = fmaxf(top, mx[c]);
+  if (!__any_sync(0xffffffffu, top > thr)) return;  // more than half of the slices of a large sweep
   uint32_t hit = 0;
 #pragma unroll
   for (int c = 0; c < kChunks; ++c) hit |= (__any_sync(0xffffffffu, mx[c] > thr) ? 1u : 0u) << c;
-  if (hit == 0) return;
 #pragma unroll
   for (int c = 0; c < kChunks; ++c)
     if (hit & (1u << c)) L.push(r[c], mx[c], jb + (uint32_t)(c * 16), n, i);
@@ -594,12 +597,12 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 // query rows and half (128) of a tile's keys, so that per MMA an SM reads
 // 8 KB and writes 4 KB, and the key bytes that come from L2 halve.
 //
-// Measured (the contraction with its row preparation, one CTA a sweep before,
-// the pair now): 72 -> 46.0 ms at n = 600,000, d = 100 (bound by the MMAs'
-// power draw and the list work; 41 ms without the list work); 6.9 -> 5.2 ms
-// at n = 100,000, d = 500 (MMA bound: 4150 cycles a tile for 32 MMAs, SM clock
-// 1.8 GHz under power); E4M3 3.4 -> 2.55 ms at n = 100,003, d = 256 (list
-// work: 1.7 ms without it).
+// Measured (the contraction with its row preparation; one CTA a sweep before,
+// the pair now): 72 -> 46 ms at n = 600,000, d = 100 (about 1240 cycles a tile
+// for 907 of MMAs: the epilogue's list work; 41 ms without it, the clock then
+// lower under power); 6.9 -> 5.2 ms at n = 100,000, d = 500 (MMA bound: 4150
+// cycles a tile for 32 MMAs, SM clock 1.8 GHz under power); E4M3 3.4 -> 2.5 ms
+// at n = 100,003, d = 256 (list work: 1.7 ms without it).
 //
 // Roles as in k_knn_tc, in both CTAs, except that the even CTA (the leader)
 // alone issues the MMAs.  Each CTA's producer loads its own half and signals
@@ -684,14 +687,17 @@ __device__ __forceinline__ void pair_arrive(uint32_t bar) {
 // rows is swept once per share of the key tiles (tiles share, share + shares,
 // ...; past the last one the keys are padding), and row i leaves two lists per
 // share, at (i * shares + share) * kCandC; qblocks counts (block, share) pairs.
-template <bool kE4M3>
+// kShared: shares may exceed 1 (as a run-time value everywhere its arithmetic
+// in the roles' loops cost 9% at d = 100: 194 against 178 ms at n = 1,200,000).
+template <bool kE4M3, bool kShared>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
 k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
            int64_t n_pad, int64_t qblocks, int kb_count, int k_last, int nstages, float* __restrict__ cand_val,
            int32_t* __restrict__ cand_idx, const float* __restrict__ out_scale, float* __restrict__ part_val,
-           int32_t* __restrict__ part_idx, const int32_t* __restrict__ a_rows, int64_t n_rows, int shares,
+           int32_t* __restrict__ part_idx, const int32_t* __restrict__ a_rows, int64_t n_rows, int share_count,
            unsigned long long* __restrict__ tick, int* __restrict__ err) {
   constexpr int kTK = kE4M3 ? 128 : 64;  // features per stage
+  const int shares = kShared ? share_count : 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -1530,8 +1536,11 @@ ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap
   ANCKA_TRY(ws.alloc(&part_val, (size_t)pairs * 2 * kPairRows * kCandC));
   ANCKA_TRY(ws.alloc(&part_idx, (size_t)pairs * 2 * kPairRows * kCandC));
   ANCKA_TRY(ws.zeros(&tick, 1));
-  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_pair<kE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_knn_pair<kE4M3><<<(unsigned)(2 * pairs), kTcThreads, smem, s>>>(
+  auto kernel = k_knn_pair<kE4M3, false>;
+  if constexpr (!kE4M3)
+    if (shares > 1) kernel = k_knn_pair<kE4M3, true>;
+  ANCKA_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kernel<<<(unsigned)(2 * pairs), kTcThreads, smem, s>>>(
       ta, tb, n, n_pad, qblocks, kb_count, k_last, nstages, cand_val, cand_idx, out_scale, part_val, part_idx,
       a_rows, n_rows, shares, tick, err);
   ANCKA_LAUNCHED();
