@@ -957,16 +957,18 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
 
 // Lists of the query blocks split between runs: per row and column half, the
 // 16 best of the pieces' lists (each piece holds the best of its own key
-// tiles, so the result is the best of the whole half).  One CTA per query
-// block, one thread per row (kRows: 128, or 256 for pairs) and half; blocks
-// that one run covered return at once.  A piece's 16 entries are loaded
-// together: with one entry at a time and both halves in one thread, the eight
-// pieces a block has at n = 2000 took 80 us of a call of 185 us.
+// tiles, so the result is the best of the whole half).  A thread
+// per row (kRows: 128, or 256 for pairs) and half; blocks that one run covered
+// return at once.  A piece's 16 entries are loaded together, and a block's
+// threads are spread over CTAs of 128: with one entry at a time, both halves in
+// one thread and a CTA per block, the eight pieces a block has at n = 2000 took
+// 80 us of a call of 185 us.
 // Block qb's work items are [x0, x1) = [qb n_tiles, (qb + 1) n_tiles), or
 // [blk_ptr[qb], blk_ptr[qb + 1]) in tile-list mode (a block with no tiles
 // gets empty lists).
+constexpr int kMergeThreads = 128;
 template <int kRows>
-__global__ void __launch_bounds__(2 * kRows)
+__global__ void __launch_bounds__(kMergeThreads)
 k_merge_lists(int n_tiles, int64_t work, int64_t ctas, const int64_t* __restrict__ blk_ptr,
               const float* __restrict__ part_val, const int32_t* __restrict__ part_idx,
               const int32_t* __restrict__ a_rows, int64_t n_rows, int shares, float* __restrict__ cand_val,
@@ -975,7 +977,8 @@ k_merge_lists(int n_tiles, int64_t work, int64_t ctas, const int64_t* __restrict
   const int64_t qb = blockIdx.x;
   const int64_t x0 = blk_ptr ? blk_ptr[qb] : qb * n_tiles;
   const int64_t x1 = blk_ptr ? blk_ptr[qb + 1] : x0 + n_tiles;
-  const int r = threadIdx.x % kRows, h = threadIdx.x / kRows;
+  const int t = blockIdx.y * kMergeThreads + threadIdx.x;
+  const int r = t % kRows, h = t / kRows;
   const int64_t ra = qb / shares * kRows + r;
   if (ra >= n_rows) return;
   const int64_t i = (a_rows ? (int64_t)a_rows[ra] : ra) * shares + qb % shares;  // the lists' row
@@ -989,24 +992,28 @@ k_merge_lists(int n_tiles, int64_t work, int64_t ctas, const int64_t* __restrict
     lv[c] = -INFINITY;
     li[c] = -1;
   }
+  // the list run cc left for the block
+  auto load = [&](int64_t cc, float (&v)[C], int32_t (&j)[C]) {
+    const int64_t b = range_begin(cc, work, ctas);
+    const int64_t slot = (cc * 2 + (b >= x0 ? 0 : 1)) * kRows + r;  // run cc starts inside the block: its first segment
+    const float4* pv = reinterpret_cast<const float4*>(part_val + slot * kCandC + h * C);
+    const int4* pi = reinterpret_cast<const int4*>(part_idx + slot * kCandC + h * C);
+#pragma unroll
+    for (int q = 0; q < C / 4; ++q) {
+      const float4 f = pv[q];
+      const int4 g = pi[q];
+      v[4 * q] = f.x, v[4 * q + 1] = f.y, v[4 * q + 2] = f.z, v[4 * q + 3] = f.w;
+      j[4 * q] = g.x, j[4 * q + 1] = g.y, j[4 * q + 2] = g.z, j[4 * q + 3] = g.w;
+    }
+  };
   if (x0 < x1) {
     const int64_t c0 = ((x0 + 1) * ctas + work - 1) / work - 1;  // the CTA whose range holds x0
     if (range_begin(c0 + 1, work, ctas) >= x1) return;           // covered whole: its lists are final
-    for (int64_t cc = c0; cc < ctas; ++cc) {
-      const int64_t b = range_begin(cc, work, ctas);
-      if (b >= x1) break;
-      const int64_t slot = (cc * 2 + (b >= x0 ? 0 : 1)) * kRows + r;  // run cc starts inside the block: its first segment
-      const float4* pv = reinterpret_cast<const float4*>(part_val + slot * kCandC + h * C);
-      const int4* pi = reinterpret_cast<const int4*>(part_idx + slot * kCandC + h * C);
+    load(c0, lv, li);  // the first piece is the list so far
+    for (int64_t cc = c0 + 1; cc < ctas && range_begin(cc, work, ctas) < x1; ++cc) {
       float v[C];
       int32_t j[C];
-#pragma unroll
-      for (int q = 0; q < C / 4; ++q) {
-        const float4 f = pv[q];
-        const int4 g = pi[q];
-        v[4 * q] = f.x, v[4 * q + 1] = f.y, v[4 * q + 2] = f.z, v[4 * q + 3] = f.w;
-        j[4 * q] = g.x, j[4 * q + 1] = g.y, j[4 * q + 2] = g.z, j[4 * q + 3] = g.w;
-      }
+      load(cc, v, j);
       // the piece is sorted: nothing after its first entry that does not pass can pass
 #pragma unroll
       for (int e = 0; e < C; ++e) {
@@ -1500,7 +1507,7 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
                                                                    out_scale, part_val, part_idx, ca, tick, err);
   ANCKA_LAUNCHED();
   if (!kCollect) {
-    k_merge_lists<kTM><<<(unsigned)qblocks, 2 * kTM, 0, s>>>(n_tiles, work, ctas, ca.blk_ptr, part_val, part_idx, ca.a_rows,
+    k_merge_lists<kTM><<<dim3((unsigned)qblocks, 2 * kTM / kMergeThreads), kMergeThreads, 0, s>>>(n_tiles, work, ctas, ca.blk_ptr, part_val, part_idx, ca.a_rows,
                                                     n_rows, 1, cand_val, cand_idx);
     ANCKA_LAUNCHED();
   }
@@ -1544,7 +1551,7 @@ ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap
       ta, tb, n, n_pad, qblocks, kb_count, k_last, nstages, cand_val, cand_idx, out_scale, part_val, part_idx,
       a_rows, n_rows, shares, tick, err);
   ANCKA_LAUNCHED();
-  k_merge_lists<kPairRows><<<(unsigned)qblocks, 2 * kPairRows, 0, s>>>(n_tiles, work, pairs, nullptr, part_val, part_idx,
+  k_merge_lists<kPairRows><<<dim3((unsigned)qblocks, 2 * kPairRows / kMergeThreads), kMergeThreads, 0, s>>>(n_tiles, work, pairs, nullptr, part_val, part_idx,
                                                                    a_rows, n_rows, shares, cand_val, cand_idx);
   ANCKA_LAUNCHED();
   return ANCKA_OK;
