@@ -583,7 +583,7 @@ def main():
         t_full = recorded_traffic(TRAFFIC_FILE, f"k_knn_tc:{args.workload}:{prec}", "knn_tc.cu")
         roof = {"bound": "tensor", "achieved": round(achieved, 2), "peak": peak, "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4), "traffic": t_full,
-                "kernel": f"k_knn_tc (tcgen05 {prec.upper()} contraction + fused top-16 x 2 lists per row)",
+                "kernel": f"k_knn_pair (tcgen05 {prec.upper()} contraction + fused top-16 x 2 lists per row)",
                 "peak_source": (f"{'bf16_tflops_sustained' if sustained else 'bf16_tflops'} of {peak_src} "
                                 f"MEASURED_PEAKS.json" + (" x 2 (FP8 = 2 x BF16 nominal)" if prec == "fp8" else "")
                                 + (" (the kernel runs for > 0.2 s inside the step)" if sustained else "")),
