@@ -31,7 +31,7 @@ namespace {
 
 // Rows per chunk of the counting sort: a warp places a chunk 32 rows at a
 // time, so short chunks put more warps to work; the chunks' table of nlist
-// positions each stays below about 4 bytes a row and 32 MB per 2^20 rows.
+// positions each takes at most 4 bytes a row up to 1024 cells and 8 at 8192.
 inline int ivf_chunk(int nlist) { return nlist <= 1024 ? 1024 : 4096; }
 constexpr int kTileRows = 256;   // key rows per tile of the contraction
 constexpr int kBlockRows = 128;  // query rows per block of the contraction
