@@ -632,14 +632,24 @@ __global__ void k_exh_merge(const int32_t* __restrict__ rows, const int32_t* __r
 // ---------------------------------------------------------------------------
 
 // thr[i] = (K-th largest lower bound of row i's per candidates) - m_max, or
-// -inf when there are fewer than K (every key is collected); one warp per row
+// -inf when there are fewer than K (every key is collected); one warp per row.
+// After a failed list pass the lists hold whatever their memory held before,
+// and are not read: thr[i] = +inf, so that the collect pass finds no key, and
+// k_rerank_wide sends the rows on.
 __global__ void __launch_bounds__(kWarps * 32)
 k_wide_threshold(const float* __restrict__ cand_val, const int32_t* __restrict__ cand_idx, int per, int64_t n, int K,
                  const float* __restrict__ err, const float* __restrict__ err_max_p, float acc,
-                 int32_t* __restrict__ rows, float* __restrict__ thr) {
+                 const int32_t* __restrict__ list_err, int32_t* __restrict__ rows, float* __restrict__ thr) {
   const int lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
   if (i >= n) return;
+  if (*list_err) {
+    if (lane == 0) {
+      rows[i] = (int32_t)i;
+      thr[i] = INFINITY;
+    }
+    return;
+  }
   const float ei = err[i], emax = *err_max_p;
   uint32_t key[4];  // 0: no candidate (below every number's key)
   int nvalid = 0;
@@ -916,7 +926,7 @@ ancka_status knn_wide(Workspace& ws, const float* X, int64_t n, int32_t d, int32
   ANCKA_LAUNCHED();
   ANCKA_TRY(knn_candidates_bf16_shares(ws, pr, n, shares, cv, ci, errs, s));
   k_wide_threshold<<<(unsigned)ceil_div(n, kWarps), kWarps * 32, 0, s>>>(cv, ci, per, n, K, pr.err, pr.err_max, acc,
-                                                                         rows, thr);
+                                                                         errs, rows, thr);
   ANCKA_LAUNCHED();
   // the collected keys of kChunk rows at a time: 2 GB of buffer at most
   constexpr int64_t kChunk = 1 << 18;
