@@ -56,11 +56,19 @@ __global__ void k_ivf_init_centroids(const __nv_bfloat16* __restrict__ xb, int d
   for (int f = threadIdx.x; f < dp; f += blockDim.x) C[(int64_t)c * dp + f] = xb[row * dp + f];
 }
 
-// the m best of a row's two sorted 16-entry lists (score desc, index asc)
+// the m best of a row's two sorted 16-entry lists (score desc, index asc);
+// -1 (no cell) for every row once a list pass has failed: its lists hold
+// whatever their memory held before, and what follows indexes with cells until
+// the host reads list_err
 __global__ void k_ivf_top(const float* __restrict__ cand_val, const int32_t* __restrict__ cand_idx,
-                          const int32_t* __restrict__ rows, int64_t n_rows, int m, int32_t* __restrict__ out) {
+                          const int32_t* __restrict__ rows, int64_t n_rows, int m, const int32_t* __restrict__ list_err,
+                          int32_t* __restrict__ out) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n_rows) return;
+  if (*list_err) {
+    for (int e = 0; e < m; ++e) out[q * m + e] = -1;
+    return;
+  }
   const int64_t i = rows ? rows[q] : q;
   const float* v = cand_val + i * kCandC;
   const int32_t* x = cand_idx + i * kCandC;
@@ -307,7 +315,8 @@ constexpr int kIvfSeg = 32;  // features per step; rows of 33 floats keep the la
 __global__ void __launch_bounds__(kIvfWarps * 32)
 k_ivf_rerank(const float* __restrict__ X, int d, const double* __restrict__ nrm2, const int32_t* __restrict__ order,
              int64_t n, const float* __restrict__ cand_val, const int32_t* __restrict__ cand_idx, int K,
-             int32_t* __restrict__ out_idx, float* __restrict__ out_sim) {
+             const int32_t* __restrict__ list_err, int32_t* __restrict__ out_idx, float* __restrict__ out_sim) {
+  if (*list_err) return;  // a list pass failed: the candidates are not valid
   __shared__ float seg[kIvfWarps][32][kIvfSeg + 1];
   const int64_t p = (int64_t)blockIdx.x * kIvfWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -474,7 +483,8 @@ ancka_status knn_ivf(Workspace& ws, const float* X, int64_t n, int32_t d, int32_
   for (int it = 0; it < iters; ++it) {
     ANCKA_TRY(knn_lists_bf16(ws, pr.xb, pr.n_pad, n_train < n ? train_rows : nullptr, n_train, C, nlist, nl_pad, dp, d,
                              nullptr, nullptr, 0, true, cv, ci, terr, s));
-    k_ivf_top<<<grid_for(n_train, 256), 256, 0, s>>>(cv, ci, n_train < n ? train_rows : nullptr, n_train, 1, cell);
+    k_ivf_top<<<grid_for(n_train, 256), 256, 0, s>>>(cv, ci, n_train < n ? train_rows : nullptr, n_train, 1, terr,
+                                                    cell);
     ANCKA_LAUNCHED();
     ANCKA_TRY(sort_by_cell(ws, cell, nullptr, n_train, nlist, order, cell_off, s));
     k_ivf_map_order<<<grid_for(n_train, 256), 256, 0, s>>>(n_train < n ? train_rows : nullptr, n_train, order);
@@ -487,7 +497,7 @@ ancka_status knn_ivf(Workspace& ws, const float* X, int64_t n, int32_t d, int32_
   ANCKA_TRY(ws.alloc(&probes, (size_t)n * nprobe));
   ANCKA_TRY(knn_lists_bf16(ws, pr.xb, pr.n_pad, nullptr, n, C, nlist, nl_pad, dp, d, nullptr, nullptr, 0, true, cv, ci,
                            terr, s));
-  k_ivf_top<<<grid_for(n, 256), 256, 0, s>>>(cv, ci, nullptr, n, nprobe, probes);
+  k_ivf_top<<<grid_for(n, 256), 256, 0, s>>>(cv, ci, nullptr, n, nprobe, terr, probes);
   ANCKA_LAUNCHED();
   k_ivf_first<<<grid_for(n, 256), 256, 0, s>>>(probes, nprobe, n, cell);
   ANCKA_LAUNCHED();
@@ -541,7 +551,8 @@ ancka_status knn_ivf(Workspace& ws, const float* X, int64_t n, int32_t d, int32_
   ANCKA_TRY(knn_lists_bf16(ws, xs, pr.n_pad, nullptr, n, xs, n, pr.n_pad, dp, d, blk_ptr, blk_tiles, work, false, cv,
                            ci, terr, s));
   // 6. exact cosines of the candidates, back to the original order
-  k_ivf_rerank<<<grid_for(n, kIvfWarps), kIvfWarps * 32, 0, s>>>(X, d, pr.nrm2, order, n, cv, ci, K, out_idx, out_sim);
+  k_ivf_rerank<<<grid_for(n, kIvfWarps), kIvfWarps * 32, 0, s>>>(X, d, pr.nrm2, order, n, cv, ci, K, terr, out_idx,
+                                                                 out_sim);
   ANCKA_LAUNCHED();
   int32_t he = 0;
   ANCKA_CUDA(cudaMemcpyAsync(&he, terr, sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -37,7 +37,7 @@ ancka_status knn_candidates_bf16_shares(Workspace& ws, const PrepOut& pr, int64_
   return real_candidates_bf16_shares(ws, pr, n, shares, cand_val, cand_idx, err, s);
 }
 
-// n_rows lists, at their own rows or at the rows given: the inverted lists' buffers hold a list for every row of a
+// the buffers hold n_rows lists at least
 ancka_status knn_lists_bf16(Workspace& ws, const __nv_bfloat16* a, int64_t a_rows_total, const int32_t* rows,
                             int64_t n_rows, const __nv_bfloat16* keys, int64_t n_keys, int64_t keys_pad, int dp, int d,
                             const int64_t* blk_ptr, const int32_t* blk_tiles, int64_t blk_work, bool no_self,

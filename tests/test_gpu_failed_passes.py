@@ -66,3 +66,22 @@ def test_narrow_lists_without_their_pass(lib):
     st, idx, sim = _knn(lib, Xd, 10, 0)
     assert st == 0
     compare_knn(X, 10, np.arange(0, 900, 7), idx.cpu().numpy(), sim.cpu().numpy())
+
+
+@pytest.mark.parametrize("n,d,nlist,nprobe", [(1500, 40, 7, 3), (9000, 20, 1025, 16)])
+@pytest.mark.parametrize("nth", [1, 8, 9, 10])  # the first and last round of the cells, the probes, the tile lists
+def test_inverted_lists_without_their_pass(lib, n, d, nlist, nprobe, nth):
+    """The status says so, every index on the way stays in range, and the next call is right."""
+    from paper_2408_05459_gb300 import ancka
+    K = 6
+    X = torch.as_tensor(np.random.default_rng(n).standard_normal((n, d)).astype(np.float32), device="cuda")
+    ref, ref_sim, _ = ancka.knn_ivf(X, K, nlist, nprobe)
+    idx = torch.empty((n, K), dtype=torch.int32, device="cuda")
+    sim = torch.empty((n, K), device="cuda")
+    for fail, status in ((nth, 5), (0, 0)):
+        lib.set_failing_pass(fail)
+        assert lib.ancka_knn_ivf(ancka._ptr(X), n, d, K, nlist, nprobe, ancka._ptr(idx), ancka._ptr(sim), None,
+                                 ancka._stream()) == status
+        lib.set_failing_pass(0)
+        torch.cuda.synchronize()
+    assert torch.equal(idx, ref) and torch.equal(sim, ref_sim)
