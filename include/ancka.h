@@ -214,6 +214,9 @@ void ancka_set_symmetric_knn_min_rows(int64_t n_min);
  *            or FP8-E4M3 (tensor cores, d <= 512).  The result is the same
  *            exact list for every precision; FP8 rows whose candidates cannot
  *            be certified are redone from BF16 candidates.
+ * An expired wait in the contraction gives ANCKA_ERR_TIMEOUT, except that a
+ * call with K > 12 (FP32: > 16) and info == NULL, which reads nothing back,
+ * recomputes its rows by the exhaustive scan: the same lists, later.
  * Requires 1 <= K <= 64, K < n, 1 <= d <= 4096, n < 2^31. */
 ancka_status ancka_knn(const float* X, int64_t n, int32_t d, int32_t K, int32_t prec,
                        int32_t* out_idx, float* out_sim, ancka_info* info, void* stream);

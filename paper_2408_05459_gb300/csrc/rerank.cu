@@ -900,8 +900,9 @@ ancka_status knn_rerank(Workspace& ws, const float* X, int64_t n, int32_t d, int
   return ANCKA_OK;
 }
 
-// Exact lists of K > the lists' certificate.  No host read: a failed pass
-// sends its rows to the exhaustive kernels on the device.
+// Exact lists of K > the lists' certificate.  A failed pass sends its rows to
+// the exhaustive kernels on the device, so that without want_counts nothing is
+// read back; with it the failure is read with the counts and reported.
 ancka_status knn_wide(Workspace& ws, const float* X, int64_t n, int32_t d, int32_t K, const PrepOut& pr, float acc,
                       int32_t* out_idx, float* out_sim, int64_t* n_fallback, int64_t* n_exhaustive, bool want_counts,
                       cudaStream_t s) {
@@ -953,9 +954,15 @@ ancka_status knn_wide(Workspace& ws, const float* X, int64_t n, int32_t d, int32
   k_knn_exhaustive<<<304, kExWarps * 32, 0, s>>>(X, n, d, K, rinv, ov_rows, ov_count, 0, out_idx, out_sim);
   ANCKA_LAUNCHED();
   if (want_counts) {
-    int32_t ex = 0;
+    int32_t ex = 0, he[2] = {0, 0};
     ANCKA_CUDA(cudaMemcpyAsync(&ex, ov_count, sizeof(ex), cudaMemcpyDeviceToHost, s));
+    ANCKA_CUDA(cudaMemcpyAsync(he, errs, sizeof(he), cudaMemcpyDeviceToHost, s));
     ANCKA_CUDA(cudaStreamSynchronize(s));
+    if (he[0] || he[1]) {
+      set_error("tensor-core %s pass: a pipeline wait expired (role %d)", he[0] ? "list" : "collect",
+                he[0] ? he[0] : he[1]);
+      return ANCKA_ERR_TIMEOUT;
+    }
     *n_fallback = n;
     if (n_exhaustive) *n_exhaustive = ex;
   }

@@ -58,6 +58,19 @@ def test_wide_lists_without_their_pass(lib, n, d, K, nth):
     compare_knn(X, K, np.arange(0, n, 7), idx.cpu().numpy(), sim.cpu().numpy())
 
 
+@pytest.mark.parametrize("nth", [1, 2])
+def test_wide_lists_report_their_pass(lib, nth):
+    """K > 12 with info, which the call reads back: the status says so, and the next call works."""
+    from paper_2408_05459_gb300 import ancka
+    X = np.random.default_rng(nth).standard_normal((700, 40)).astype(np.float32)
+    Xd = torch.as_tensor(X, device="cuda")
+    assert _knn(lib, Xd, 20, nth, ancka.Info())[0] == 5  # ANCKA_ERR_TIMEOUT
+    info = ancka.Info()
+    st, idx, sim = _knn(lib, Xd, 20, 0, info)
+    assert st == 0 and info.knn_exhaustive_rows == 0
+    compare_knn(X, 20, np.arange(0, 700, 7), idx.cpu().numpy(), sim.cpu().numpy())
+
+
 def test_narrow_lists_without_their_pass(lib):
     """K <= 12: the status says so, and the next call works."""
     X = np.random.default_rng(5).standard_normal((900, 64)).astype(np.float32)
