@@ -193,7 +193,11 @@ struct RowList {
 
 // Collect mode: append every key whose score reaches the row's fixed
 // threshold t to the row's buffer (cap entries; the counter keeps counting
-// past cap so the caller can see an overflow).
+// past cap so the caller can see an overflow).  One atomic reserves a chunk's
+// places: with one per key, a row whose keys nearly all pass waited for 32 of
+// them in turn at every chunk, long after its buffer was full (a call at
+// n = 8000, d = 500, K = 13 with a quarter of the rows near-parallel: 2.19 ->
+// 1.91 ms).
 __device__ __forceinline__ void collect_chunk(const uint32_t (&r)[32], float mx, int64_t j0, int64_t n, int64_t i,
                                               float t, int64_t ra, int32_t* __restrict__ cnt,
                                               int32_t* __restrict__ buf, int cap) {
@@ -203,11 +207,10 @@ __device__ __forceinline__ void collect_chunk(const uint32_t (&r)[32], float mx,
   for (int e = 0; e < 32; ++e) pm |= (__uint_as_float(r[e]) >= t ? 1u : 0u) << e;
   if (j0 + 32 > n) pm &= (j0 >= n) ? 0u : ((1u << (uint32_t)(n - j0)) - 1u);
   if (i >= j0 && i < j0 + 32) pm &= ~(1u << (uint32_t)(i - j0));
-  while (pm) {
-    const int e = __ffs(pm) - 1;
+  if (!pm) return;
+  for (int pos = atomicAdd(&cnt[ra], __popc(pm)); pm && pos < cap; ++pos) {
+    buf[ra * (int64_t)cap + pos] = (int32_t)(j0 + __ffs(pm) - 1);
     pm &= pm - 1;
-    const int pos = atomicAdd(&cnt[ra], 1);
-    if (pos < cap) buf[ra * (int64_t)cap + pos] = (int32_t)(j0 + e);
   }
 }
 
