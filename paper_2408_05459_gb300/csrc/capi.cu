@@ -217,6 +217,14 @@ float tc_acc_bound(int dp, int k_per_mma, int ulp_log2) {
   return (float)((dp / k_per_mma + 2) * std::ldexp(1.0, ulp_log2));
 }
 
+// The exhaustive scan of a few rows (a CTA per row, so with up to 152 rows one
+// per SM; its time grows with rows an SM and with K, whose inserts are FP64)
+// ends before the wide path's dozen launches do.  Microseconds a call, scan /
+// wide path, d = 32: n = 40, K = 20: 46 / 89; n = 100: K = 13: 51 / 78, K = 40:
+// 98 / 107, K = 64: 141 / 107; n = 152, K = 50: 141 / 147; n = 160: K = 13:
+// 78 / 89, K = 16: 90 / 86; n = 200, K = 16: 102 / 89.  d changes both little.
+bool scan_is_short(int64_t n, int32_t K) { return n * K <= 2600 || (n <= 152 && K <= 50); }
+
 // the KNN lists with every step on the device
 // after_contraction (may be empty): called once the contraction kernel is
 // enqueued, before the first host read (with device inputs the cluster call
@@ -229,8 +237,9 @@ ancka_status knn_impl(Workspace& ws, const float* X, int64_t n, int32_t d, int32
   // K beyond what two lists certify: the wide path, whatever the precision
   // asked for (the lists are exact); it keeps the query block of the BF16
   // contraction in shared memory.  An exhaustive FP32 scan of every pair, the
-  // route left for larger d, took 11.1 ms at n = 3001, d = 500, K = 50.
-  const bool wide = K > max_candidate_K(prec) && round_up(d, 64) <= knn_tc_max_dp();
+  // route left for larger d and for a few rows, took 11.1 ms at n = 3001,
+  // d = 500, K = 50.
+  const bool wide = K > max_candidate_K(prec) && round_up(d, 64) <= knn_tc_max_dp() && !scan_is_short(n, K);
   PrepOut pr;
   ANCKA_TRY(prep_rows(ws, X, n, d, wide ? ANCKA_PREC_BF16 : prec, &pr, s));
   if (zero_row) *zero_row = pr.zero_row;
