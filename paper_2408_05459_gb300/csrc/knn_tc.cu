@@ -62,7 +62,10 @@ constexpr int kABytes = kTM * kTKB;      // 16 KB per 128-byte block of A
 constexpr int kBBytes = kTN * kTKB;      // 32 KB per stage of B
 constexpr int kMmaPerStage = 4;          // 32 bytes of K per MMA: 16 BF16 or 32 FP8
 constexpr int kMaxStages = 8;
-constexpr int kMaxSmem = 232448;         // 227 KB opt-in dynamic shared memory
+// 227 KB opt-in dynamic shared memory; every kernel's limit is set to it,
+// whatever the call needs, since the limit is the process's and another
+// thread's call may need more
+constexpr int kMaxSmem = 232448;
 constexpr uint32_t kTmemCols = 512;      // two 256-column FP32 accumulators
 
 // instruction descriptors: D = F32 (bits 4-5 = 1), both operands K-major,
@@ -1504,7 +1507,7 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
   // on every call: a key order that moves with timing resolves exact score
   // ties differently)
   if (key_stride == 1 && !ca.blk_ptr && !ca.no_self) ANCKA_TRY(ws.zeros(&tick, 1));
-  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_tc<kCollect>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_tc<kCollect>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   k_knn_tc<kCollect><<<(unsigned)ctas, kTcThreads, smem, s>>>(ta, tb, n, n_pad, qblocks, kb_count, k_last,
                                                                    nstages, key_stride, cand_val, cand_idx,
                                                                    out_scale, part_val, part_idx, ca, tick, err);
@@ -1549,7 +1552,7 @@ ancka_status launch_pair(Workspace& ws, const CUtensorMap& ta, const CUtensorMap
   auto kernel = k_knn_pair<kE4M3, false>;
   if constexpr (!kE4M3)
     if (shares > 1) kernel = k_knn_pair<kE4M3, true>;
-  ANCKA_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ANCKA_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   kernel<<<(unsigned)(2 * pairs), kTcThreads, smem, s>>>(
       ta, tb, n, n_pad, qblocks, kb_count, k_last, nstages, cand_val, cand_idx, out_scale, part_val, part_idx,
       a_rows, n_rows, shares, tick, err);
@@ -1616,7 +1619,7 @@ ancka_status knn_candidates_bf16_sym(Workspace& ws, const PrepOut& pr, int64_t n
   const int64_t qblocks = ceil_div(n, kTM);
   const int64_t work = sym_start_host(qblocks, n_tiles);
   const int64_t ctas = std::min<int64_t>(sms, work);
-  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ANCKA_CUDA(cudaFuncSetAttribute(k_knn_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   k_knn_sym<<<(unsigned)ctas, kThreads, smem, s>>>(ta, tb, n, pr.n_pad, qblocks, kb_count, nstages, sa, err);
   ANCKA_LAUNCHED();
   // 4. staged entries into the row-half buffers, then the two lists of every row

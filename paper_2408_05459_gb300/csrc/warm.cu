@@ -27,6 +27,7 @@ namespace ancka {
 namespace {
 
 constexpr int kHidden = 256;
+constexpr int kWarmMaxK = 64;
 
 __global__ void k_unit_rows(const float* __restrict__ X, int64_t n, int d, int ld, float* __restrict__ U) {
   const int lane = threadIdx.x & 31;
@@ -527,7 +528,9 @@ ancka_status warm_forward(Workspace& ws, const __nv_bfloat16* A, int64_t n, int 
   if (!H) ANCKA_TRY(ws.alloc(&H, (size_t)n * kHidden));
   ANCKA_TRY(gemm_bias_gelu(A, n, kp, W1t, b1, Z1, H, kHidden, err, s));
   const size_t smem = (size_t)kHidden * k * sizeof(float);
-  ANCKA_CUDA(cudaFuncSetAttribute(k_mlp_out, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (limits are the process's: those of k = 64, as other threads' calls may need them)
+  ANCKA_CUDA(cudaFuncSetAttribute(k_mlp_out, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(kHidden * kWarmMaxK * sizeof(float))));
   // at most three CTAs an SM at k = 64 (64 KB each), so four waves at most
   k_mlp_out<<<(unsigned)std::min<int64_t>(ceil_div(n, 8), 152 * 6), 256, smem, s>>>(H, n, W2, b2, k, W, ldw);
   ANCKA_LAUNCHED();
@@ -572,7 +575,8 @@ ancka_status warm_train_step(Workspace& ws, const WarmStepArgs& a, cudaStream_t 
   ANCKA_TRY(xty(ws, W, ldw, W, ldw, n, k, k, G, s));
   ANCKA_TRY(xty(ws, a.Qt, a.ldq, W, ldw, n, k, k, M, s));
   const size_t csm = (size_t)5 * k * k * sizeof(double);
-  ANCKA_CUDA(cudaFuncSetAttribute(k_warm_coeffs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+  ANCKA_CUDA(cudaFuncSetAttribute(k_warm_coeffs, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(5 * kWarmMaxK * kWarmMaxK * sizeof(double))));
   k_warm_coeffs<<<1, kCoeffThreads, csm, s>>>(G, M, k, (double)n, (double)a.lam, C1, C2, a.loss_dev, a.status);
   ANCKA_LAUNCHED();
   k_grad_w<<<(unsigned)ceil_div(n * k, 256), 256, (size_t)2 * k * k * sizeof(float), s>>>(W, ldw, a.Qt, a.ldq, n, k,
