@@ -55,3 +55,23 @@ def test_overflowing_rows_cost_the_scan_they_end_in():
     assert best(X) <= 1.06 * best(wider)
     _, _, info = ancka.knn(X, K, "bf16")
     assert info["knn_exhaustive_rows"] == n
+
+
+def test_more_rows_than_one_collect_pass():
+    """The collected keys are taken 2^18 rows at a time: rows on both sides of the second pass's first one and the
+    last rows, with copies across it."""
+    from tests.parity_util import compare_knn
+
+    from paper_2408_05459_gb300 import ancka
+    step = 1 << 18
+    n, d, K = step + 131, 16, 13
+    X = np.random.default_rng(2).standard_normal((n, d)).astype(np.float32)
+    X[step] = X[step - 1]
+    X[n - 1] = X[3]
+    X[step + 5] = 0.0
+    idx, sim, info = ancka.knn(torch.as_tensor(X, device="cuda"), K, "bf16")
+    torch.cuda.synchronize()
+    rows = np.r_[0:6, step // 2:step // 2 + 3, step - 4:step + 5, step + 6:step + 10, step + 120:n]
+    compare_knn(X, K, rows, idx.cpu().numpy(), sim.cpu().numpy())
+    assert idx[step + 5].tolist() == list(range(K))  # a zero row: the lowest indices
+    assert info["knn_exhaustive_rows"] >= 1
