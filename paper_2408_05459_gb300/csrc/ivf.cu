@@ -532,9 +532,7 @@ ancka_status knn_ivf(Workspace& ws, const float* X, int64_t n, int32_t d, int32_
   int64_t *blk_cnt, *blk_ptr;
   ANCKA_TRY(ws.alloc(&blk_cnt, (size_t)qblocks));
   ANCKA_TRY(ws.alloc(&blk_ptr, (size_t)qblocks + 1));
-  const size_t bm = (size_t)((n_tiles + 31) / 32) * sizeof(uint32_t);
-  if (bm > 48 * 1024)
-    ANCKA_CUDA(cudaFuncSetAttribute(k_ivf_block_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bm));
+  const size_t bm = (size_t)((n_tiles + 31) / 32) * sizeof(uint32_t);  // 8 KB at most
   k_ivf_block_tiles<<<(unsigned)qblocks, kBlockRows, bm, s>>>(sprobes, nprobe, n, cell_off, n_tiles, 0, blk_cnt,
                                                               nullptr, nullptr);
   ANCKA_LAUNCHED();

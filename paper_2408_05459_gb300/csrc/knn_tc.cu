@@ -1,8 +1,9 @@
 // tcgen05 BF16 / FP8-e4m3 candidate search for the cosine KNN of Section 3.1.
 //
 // Two kernels share one scheme.  k_knn_pair sweeps all keys with CTA pairs
-// (every full sweep); k_knn_tc, one CTA at a time, takes the sweeps of listed
-// key tiles, of a sample of the tiles and of keys above a threshold.
+// (every sweep of the rows over themselves); k_knn_tc, one CTA at a time, takes
+// the sweeps of listed key tiles, of the inverted lists' centroids, of a sample
+// of the tiles and of keys above a threshold.
 //
 // Persistent CTAs (one per SM) share the (query block, 256-row key tile)
 // pairs in equal contiguous runs (stream-K), so no wave tail is left idle.
@@ -317,8 +318,7 @@ __device__ __forceinline__ int key_rotation(int64_t qb, int n_tiles, int64_t wor
 }
 
 // kCollect: collect mode (keys above a per-row threshold) instead of list
-// mode (two 16-entry lists per row).  out_scale (list
-// mode, may be null) multiplies the scores written out.
+// mode (two 16-entry lists per row).
 // key_stride > 1: only every key_stride-th key tile is swept (the sampled
 // pass of the symmetric contraction).  k_last: MMAs issued for the last
 // 128-byte block of features (those past the last one holding a feature of
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
          int64_t n_pad, int64_t qblocks, int kb_count, int k_last, int nstages, int key_stride,
          float* __restrict__ cand_val,
-         int32_t* __restrict__ cand_idx, const float* __restrict__ out_scale, float* __restrict__ part_val,
+         int32_t* __restrict__ cand_idx, float* __restrict__ part_val,
          int32_t* __restrict__ part_idx, CollectArgs ca, unsigned long long* __restrict__ tick,
          int* __restrict__ err) {
   constexpr int kTK = 64;  // features per stage
@@ -394,12 +394,14 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
           ok = false;
           break;
         }
-        // A block this CTA sweeps whole starts at the key tile the CTAs are
-        // reading now (tiles issued by all CTAs / CTAs), so that CTAs whose
-        // rates drift apart re-align at every block and keep sharing the key
-        // tiles in L2; a split block keeps the static rotation both of its
-        // CTAs can compute.
-        if (tick && !ca.blk_ptr && t0 == 0 && t1 == n_tiles)
+        // Collect mode: a block this CTA sweeps whole starts at the key tile
+        // the CTAs are reading now (tiles issued by all CTAs / CTAs), so that
+        // CTAs whose rates drift apart re-align at every block and keep
+        // sharing the key tiles in L2; a split block keeps the static rotation
+        // both of its CTAs can compute.  (Not for lists, whose callers want the
+        // same ones on every call: a key order that moves with timing resolves
+        // exact score ties differently.)
+        if (kCollect && t0 == 0 && t1 == n_tiles)
           rot = (int)((*reinterpret_cast<volatile unsigned long long*>(tick) / gridDim.x) % (uint64_t)n_tiles);
         rot = __shfl_sync(0xffffffffu, rot, 0);
         if (elect_one()) {
@@ -430,7 +432,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
               phase ^= 1;
             }
           }
-          if (tick && ((++tiles_issued) & 15) == 0 && lane == 0) atomicAdd(tick, 16ull);
+          if (kCollect && ((++tiles_issued) & 15) == 0 && lane == 0) atomicAdd(tick, 16ull);
         }
       }
       if (!ok) {  // drain this warp's copies still in flight (bounded)
@@ -506,7 +508,6 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     const int r = q * 32 + lane;
     constexpr int C = kListC;
     const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
-    const float sc = (!kCollect && out_scale) ? *out_scale : 1.f;
     int64_t g = 0;
     int seg = 0;
     bool ok = true;
@@ -578,7 +579,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         }
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          ov[h * C + c] = L.lv[c] * sc;
+          ov[h * C + c] = L.lv[c];
           oi[h * C + c] = L.li[c];
         }
       }
@@ -1479,8 +1480,7 @@ __global__ void k_gather_rows(const uint8_t* __restrict__ x, int row_bytes, cons
 template <bool kCollect>
 ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& tb, int64_t n, int64_t n_pad,
                        int64_t n_rows, int kb_count, int d, float* cand_val, int32_t* cand_idx,
-                       const float* out_scale, const CollectArgs& ca, int32_t* err, cudaStream_t s,
-                       int key_stride = 1) {
+                       const CollectArgs& ca, int32_t* err, cudaStream_t s, int key_stride = 1) {
   // MMAs over the last 128-byte feature block: K = 16 features each; the
   // padding past d is zero and needs none
   const int per_kb = 64, per_mma = 16;
@@ -1503,14 +1503,11 @@ ancka_status launch_tc(Workspace& ws, const CUtensorMap& ta, const CUtensorMap& 
     ANCKA_TRY(ws.alloc(&part_idx, (size_t)ctas * 2 * kTM * kCandC));
   }
   unsigned long long* tick = nullptr;  // tiles issued by all CTAs (re-aligns whole blocks' key order)
-  // (not for tile lists or foreign keys, whose callers want the same lists
-  // on every call: a key order that moves with timing resolves exact score
-  // ties differently)
-  if (key_stride == 1 && !ca.blk_ptr && !ca.no_self) ANCKA_TRY(ws.zeros(&tick, 1));
+  if (kCollect) ANCKA_TRY(ws.zeros(&tick, 1));
   ANCKA_CUDA(cudaFuncSetAttribute(k_knn_tc<kCollect>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   k_knn_tc<kCollect><<<(unsigned)ctas, kTcThreads, smem, s>>>(ta, tb, n, n_pad, qblocks, kb_count, k_last,
                                                                    nstages, key_stride, cand_val, cand_idx,
-                                                                   out_scale, part_val, part_idx, ca, tick, err);
+                                                                   part_val, part_idx, ca, tick, err);
   ANCKA_LAUNCHED();
   if (!kCollect) {
     k_merge_lists<kTM><<<dim3((unsigned)qblocks, 2 * kTM / kMergeThreads), kMergeThreads, 0, s>>>(n_tiles, work, ctas, ca.blk_ptr, part_val, part_idx, ca.a_rows,
@@ -1585,7 +1582,7 @@ ancka_status knn_candidates_bf16_sym(Workspace& ws, const PrepOut& pr, int64_t n
   ANCKA_TRY(ws.alloc(&sv, (size_t)n * kCandC));
   ANCKA_TRY(ws.alloc(&si, (size_t)n * kCandC));
   CollectArgs none{};
-  const ancka_status st = launch_tc<false>(ws, ta, tb, n, pr.n_pad, n, kb_count, pr.d, sv, si, nullptr, none,
+  const ancka_status st = launch_tc<false>(ws, ta, tb, n, pr.n_pad, n, kb_count, pr.d, sv, si, none,
                                                   err, s, kSymStride);
   if (st != ANCKA_OK) return st;
   // 2. thresholds
@@ -1724,8 +1721,7 @@ ancka_status knn_lists_bf16(Workspace& ws, const __nv_bfloat16* a, int64_t a_row
   ca.blk_tiles = blk_tiles;
   ca.blk_work = blk_work;
   ca.no_self = no_self ? 1 : 0;
-  return launch_tc<false>(ws, ta, tb, n_keys, keys_pad, n_rows, kb_count, d, cand_val, cand_idx, nullptr, ca,
-                                 err, s);
+  return launch_tc<false>(ws, ta, tb, n_keys, keys_pad, n_rows, kb_count, d, cand_val, cand_idx, ca, err, s);
 }
 
 ancka_status knn_collect_bf16(Workspace& ws, const PrepOut& pr, int64_t n, const int32_t* rows, int64_t n_a,
@@ -1741,7 +1737,7 @@ ancka_status knn_collect_bf16(Workspace& ws, const PrepOut& pr, int64_t n, const
   ANCKA_TRY(make_map(&ta, af, pr.dp, n_a_pad, kTM, 2));
   ANCKA_TRY(make_map(&tb, pr.xb, pr.dp, pr.n_pad, kTN, 2));
   CollectArgs ca{rows, n_a, thr, cnt, buf, cap};
-  return launch_tc<true>(ws, ta, tb, n, pr.n_pad, n_a, kb_count, pr.d, nullptr, nullptr, nullptr, ca, err, s);
+  return launch_tc<true>(ws, ta, tb, n, pr.n_pad, n_a, kb_count, pr.d, nullptr, nullptr, ca, err, s);
 }
 
 }  // namespace ancka
