@@ -531,7 +531,7 @@ ancka_status warm_forward(Workspace& ws, const __nv_bfloat16* A, int64_t n, int 
   // (limits are the process's: those of k = 64, as other threads' calls may need them)
   ANCKA_CUDA(cudaFuncSetAttribute(k_mlp_out, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)(kHidden * kWarmMaxK * sizeof(float))));
-  // at most three CTAs an SM at k = 64 (64 KB each), so four waves at most
+  // six CTAs an SM at most; at k = 64 three fit (64 KB each), so two waves
   k_mlp_out<<<(unsigned)std::min<int64_t>(ceil_div(n, 8), 152 * 6), 256, smem, s>>>(H, n, W2, b2, k, W, ldw);
   ANCKA_LAUNCHED();
   return ANCKA_OK;
@@ -592,6 +592,11 @@ ancka_status warm_train_step(Workspace& ws, const WarmStepArgs& a, cudaStream_t 
   const int nb = (int)std::min<int64_t>(304, ceil_div(n_pad, (int64_t)kDzRows));
   float2* db1p;
   ANCKA_TRY(ws.alloc(&db1p, (size_t)nb * kHidden));
+  // Five widths bound what the zero columns cost: at n = 200,000 (the kernel
+  // alone) k = 4: 183 us, 174 with an instance of its own width; k = 9: 227 and
+  // 202; k = 16: 228 and 215; k = 24: 244 and 238; k = 33: 305 and 259; k = 36:
+  // 306 and 258; k = 52: 333 and 320.  That is 1.5% of a step (3.1 ms at
+  // d = 256, k = 20) at most; all 16 widths would triple the kernel's code.
   auto dz1 = k <= 8 ? k_dz1<2> : k <= 20 ? k_dz1<5> : k <= 32 ? k_dz1<8> : k <= 48 ? k_dz1<12> : k_dz1<16>;
   dz1<<<nb, kHidden, 0, s>>>(dW, ldw, Z1, a.W2, k, n, n_pad, dZ1t, db1p);
   ANCKA_LAUNCHED();
